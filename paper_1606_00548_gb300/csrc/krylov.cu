@@ -63,11 +63,39 @@ __global__ void __launch_bounds__(512) spmv_kernel(GridDesc g, const double *__r
     spmv_row<B, X>(g, J, x, y, i);
 }
 
-// ---- block reduction of nv partial sums into partials[k][gridDim] ----------
+// ---- reductions -------------------------------------------------------------
+// The FP64 pipe takes 2 lanes per clock and SM, so a block's own reduction is
+// work to be counted like the products it follows: a five-step shuffle tree per
+// value costs 5 FP64 adds a thread and value (27 us for 29 values at three blocks
+// of 256 threads per SM, whatever the vector length).  A recursive halving over the
+// lanes costs one: at each step a lane keeps half of the values and adds its
+// partner's copy of them, and lane k ends with the warp's total of value k.
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
+}
+
+// total over the warp of a[lane] (K <= 32 values; lanes >= K return a value of no
+// meaning); a is consumed
+template <int K>
+__device__ __forceinline__ double warp_scatter_sum(double (&a)[K]) {
+    static_assert(K <= 32, "one value per lane");
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; i++) {
+            if (i + o < K) {
+                const double send = up ? a[i] : a[i + o], keep = up ? a[i + o] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            } else if (i < K) {
+                a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
+            }
+        }
+    }
+    return a[0];
 }
 
 // A block's place in the grid its reduction spans: the launch's own grid
@@ -76,22 +104,31 @@ __device__ __forceinline__ double warp_sum(double v) {
 struct VBlk { int id, count; };
 __device__ __forceinline__ VBlk grid_blk() { return VBlk{(int)blockIdx.x, (int)gridDim.x}; }
 
+// block sums of NV per-thread values over the first kRedThreads threads, into
+// partials[k][count] at the block's place
 template <int NV>
-__device__ void block_partials(const double (&acc)[NV], int nv, double *partials, VBlk vb = grid_blk()) {
-    __shared__ double sh[SIM_THREADS / 32][NV];
+__device__ void block_partials(double (&acc)[NV], double *partials, VBlk vb = grid_blk()) {
+    constexpr int LO = NV < 32 ? NV : 32;
+    __shared__ double sh[kRedThreads / 32][NV];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x < kRedThreads) {
+        double lo[LO];
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        if (k < nv) {
-            double v = warp_sum(acc[k]);
-            if (lane == 0) sh[wid][k] = v;
+        for (int k = 0; k < LO; k++) lo[k] = acc[k];
+        const double v = warp_scatter_sum<LO>(lo);
+        if (lane < LO) sh[wid][lane] = v;
+#pragma unroll
+        for (int k = LO; k < NV; k++) {
+            const double u = warp_sum(acc[k]);
+            if (lane == 0) sh[wid][k] = u;
         }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < nv; k += blockDim.x) {
+    if (threadIdx.x < NV) {
         double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += sh[w][k];
-        partials[k * vb.count + vb.id] = s;
+#pragma unroll
+        for (int w = 0; w < kRedThreads / 32; w++) s += sh[w][threadIdx.x];
+        partials[threadIdx.x * vb.count + vb.id] = s;
     }
 }
 
@@ -109,47 +146,75 @@ __device__ bool last_block(unsigned int *ticket, int count = (int)gridDim.x) {
     return last;
 }
 
-// one warp per value: lanes stride over the block partials, then a fixed
-// shuffle tree (the summation order does not depend on timing).  A lane loads
-// 8 of its partials before adding them in stride order, so the loads overlap
-// instead of each waiting for the previous add.
+// out[k] = sum of the G block partials of value k, by the whole block.  Eight lanes
+// take a value (one value: a warp), so the 32 values of a long basis are folded at
+// once and a lane's loads are all in flight before its adds; the order is fixed by
+// the lane stride and the shuffle tree, not by timing.  152 partials of 31 values:
+// 1.2 us (4.4 us with a warp per value taking its values in turn, 456 partials).
 __device__ void fold(const double *partials, int nv, double *out, int G = (int)gridDim.x) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = wid; k < nv; k += nw) {
-        const double *p = partials + (long)k * G;
+    const int L = nv > 1 ? 8 : 32;                 // lanes per value
+    const int sub = threadIdx.x & (L - 1), slots = kRedThreads / L;
+    if (threadIdx.x >= kRedThreads) return;
+    for (int k0 = 0; k0 < nv; k0 += slots) {       // uniform over the warp: the shuffles see every lane
+        const int k = k0 + threadIdx.x / L;
         double s = 0.0;
-        for (int b0 = lane; b0 < G; b0 += 32 * 8) {
-            double v[8];
+        if (k < nv) {
+            const double *p = partials + (long)k * G;
+            for (int b0 = sub; b0 < G; b0 += L * 10) {
+                double v[10];
 #pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = b0 + 32 * u < G ? __ldcg(p + b0 + 32 * u) : 0.0;
+                for (int u = 0; u < 10; u++) v[u] = b0 + L * u < G ? __ldcg(p + b0 + L * u) : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; u++)
-                if (b0 + 32 * u < G) s += v[u];
+                for (int u = 0; u < 10; u++) s += v[u];
+            }
         }
-        s = warp_sum(s);
-        if (lane == 0) out[k] = s;
+        for (int o = L >> 1; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (sub == 0 && k < nv) out[k] = s;
     }
 }
 
 constexpr int NVMAX = SIM_MAX_M + 1;
 
+// Elements of a thread's grid-stride loop taken together in the Gram-Schmidt
+// kernels: a short basis needs several elements' loads in flight (6 vectors, 3M
+// entries: 45 us against 50 us one at a time), a long one has NV loads per element
+constexpr __host__ __device__ int orth_unroll(int nv) { return nv <= 6 ? 4 : nv <= 12 ? 2 : 1; }
+
 // h[k] = V_k . w, k < NV (NV exact: no predicated work for absent vectors),
 // and h[NV] = w . w (the norm the selective reorthogonalisation test needs).
-// Above 20 vectors two blocks per SM (128 registers a thread) keep more of an
-// element's NV loads in flight than three blocks at 80 registers.
+// Bound by the FP64 pipe (NV + 1 FMAs per 8 (NV + 1) bytes): 8 to 16 warps per SM
+// keep it busy, and fewer threads leave less to reduce (sim_red_blocks).
 template <int NV>
 __device__ __forceinline__ void dots_body(const double *__restrict__ V, const double *__restrict__ w, long n,
                                           double *partials, unsigned int *ticket, double *out, VBlk vb) {
+    constexpr int U = orth_unroll(NV);
     double acc[NV + 1];
 #pragma unroll
     for (int k = 0; k <= NV; k++) acc[k] = 0.0;
-    for (long i = vb.id * (long)blockDim.x + threadIdx.x; i < n; i += (long)vb.count * blockDim.x) {
+    const long st = (long)vb.count * kRedThreads;
+    long i = vb.id * (long)kRedThreads + threadIdx.x;
+    for (; i + (U - 1) * st < n; i += U * st) {
+        double wi[U], v[U][NV];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            wi[u] = w[i + u * st];
+#pragma unroll
+            for (int k = 0; k < NV; k++) v[u][k] = V[k * n + i + u * st];
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+#pragma unroll
+            for (int k = 0; k < NV; k++) acc[k] += v[u][k] * wi[u];
+            acc[NV] += wi[u] * wi[u];
+        }
+    }
+    for (; i < n; i += st) {
         const double wi = w[i];
 #pragma unroll
         for (int k = 0; k < NV; k++) acc[k] += V[k * n + i] * wi;
         acc[NV] += wi * wi;
     }
-    block_partials<NV + 1>(acc, NV + 1, partials, vb);
+    block_partials<NV + 1>(acc, partials, vb);
     if (last_block(ticket, vb.count)) {
         fold(partials, NV + 1, out, vb.count);
         if (threadIdx.x == 0) *ticket = 0u;
@@ -157,9 +222,9 @@ __device__ __forceinline__ void dots_body(const double *__restrict__ V, const do
 }
 
 template <int NV>
-__global__ void __launch_bounds__(SIM_THREADS, NV > 20 ? 2 : 3) dots_kernel(const double *__restrict__ V, const double *__restrict__ w,
-                                                           long n, double *partials, unsigned int *ticket,
-                                                           double *out, const int *done) {
+__global__ void __launch_bounds__(kRedThreads, 2) dots_kernel(const double *__restrict__ V, const double *__restrict__ w,
+                                                              long n, double *partials, unsigned int *ticket,
+                                                              double *out, const int *done) {
     if (skip(done)) return;
     dots_body<NV>(V, w, n, partials, ticket, out, grid_blk());
 }
@@ -176,53 +241,55 @@ __device__ __forceinline__ bool need_reorth(const double *h, int nv, int selecti
 }
 
 // w -= sum_k h[k] V_k ; out[k] = V_k . w (second Gram-Schmidt pass); nothing
-// when the selective test finds no second pass is needed.  A block takes
-// tiles of 128 elements: each thread updates one element, keeping the tile's
-// basis entries in shared memory, then thread (k, sub) accumulates
-// V_k . w over the tile's elements sub, sub + 4, ... (few registers, so
-// several blocks share an SM; rows padded to 132 doubles: conflict-free).
-constexpr int kOrthTile = 128, kOrthPad = 132;
-
+// when the selective test finds no second pass is needed.  A thread keeps its
+// element's NV basis entries in registers between the update and the products, so
+// the basis is read once (2 NV FMAs per 8 (NV + 2) bytes: bound by the FP64 pipe).
 template <int NV>
 __device__ __forceinline__ void orth_dots_body(const double *__restrict__ V, double *__restrict__ w, long n,
                                                const double *h, double *partials, unsigned int *ticket, double *out,
                                                int selective, VBlk vb) {
     if (!need_reorth(h, NV, selective)) return;
-    __shared__ double sv[NV][kOrthPad];
-    __shared__ double sw[kOrthTile];
+    constexpr int U = orth_unroll(NV);
     __shared__ double hs[NV];
-    for (int k = threadIdx.x; k < NV; k += blockDim.x) hs[k] = h[k];
+    if (threadIdx.x < NV) hs[threadIdx.x] = h[threadIdx.x];
     __syncthreads();
-    const int kk = threadIdx.x >> 2, sub = threadIdx.x & 3;   // dot slot of this thread
-    double acc = 0.0;
-    for (long base = (long)vb.id * kOrthTile; base < n; base += (long)vb.count * kOrthTile) {
-        const long i = base + threadIdx.x;
-        if (i < n) {
-            double wi = w[i];
+    double acc[NV];
 #pragma unroll
-            for (int k = 0; k < NV; k++) {
-                const double v = V[k * n + i];
-                sv[k][threadIdx.x] = v;
-                wi -= hs[k] * v;
-            }
-            w[i] = wi;
-            sw[threadIdx.x] = wi;
-        } else {
+    for (int k = 0; k < NV; k++) acc[k] = 0.0;
+    const long st = (long)vb.count * kRedThreads;
+    long i = vb.id * (long)kRedThreads + threadIdx.x;
+    for (; i + (U - 1) * st < n; i += U * st) {
+        double wi[U], v[U][NV];
 #pragma unroll
-            for (int k = 0; k < NV; k++) sv[k][threadIdx.x] = 0.0;
-            sw[threadIdx.x] = 0.0;
+        for (int u = 0; u < U; u++) {
+            wi[u] = w[i + u * st];
+#pragma unroll
+            for (int k = 0; k < NV; k++) v[u][k] = V[k * n + i + u * st];
         }
-        __syncthreads();
-        if (kk < NV) {
-#pragma unroll 8
-            for (int e = sub; e < kOrthTile; e += 4) acc += sv[kk][e] * sw[e];
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            const double hk = hs[k];
+#pragma unroll
+            for (int u = 0; u < U; u++) wi[u] -= hk * v[u][k];
         }
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            w[i + u * st] = wi[u];
+#pragma unroll
+            for (int k = 0; k < NV; k++) acc[k] += v[u][k] * wi[u];
+        }
     }
-    // the 4 threads of a slot are adjacent lanes: fold them, then one per slot writes
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    if (sub == 0 && kk < NV) partials[kk * vb.count + vb.id] = acc;
+    for (; i < n; i += st) {
+        double wi = w[i], v[NV];
+#pragma unroll
+        for (int k = 0; k < NV; k++) v[k] = V[k * n + i];
+#pragma unroll
+        for (int k = 0; k < NV; k++) wi -= hs[k] * v[k];
+        w[i] = wi;
+#pragma unroll
+        for (int k = 0; k < NV; k++) acc[k] += v[k] * wi;
+    }
+    block_partials<NV>(acc, partials, vb);
     if (last_block(ticket, vb.count)) {
         fold(partials, NV, out, vb.count);
         if (threadIdx.x == 0) *ticket = 0u;
@@ -230,50 +297,71 @@ __device__ __forceinline__ void orth_dots_body(const double *__restrict__ V, dou
 }
 
 template <int NV>
-__global__ void __launch_bounds__(kOrthTile) orth_dots_kernel(const double *__restrict__ V, double *__restrict__ w,
-                                                             long n, const double *h, double *partials,
-                                                             unsigned int *ticket, double *out, const int *done,
-                                                             int selective) {
+__global__ void __launch_bounds__(kRedThreads, NV > 17 ? 1 : 2) orth_dots_kernel(const double *__restrict__ V,
+                                                                                double *__restrict__ w, long n,
+                                                                                const double *h, double *partials,
+                                                                                unsigned int *ticket, double *out,
+                                                                                const int *done, int selective) {
     if (skip(done)) return;
     orth_dots_body<NV>(V, w, n, h, partials, ticket, out, selective, grid_blk());
 }
 
 // w -= sum_k h2[k] V_k ; ||w||; last block: Hessenberg column j, Givens, test
-// (NV = j + 1 at compile time: the NV basis loads of an element are unrolled
-// and in flight together)
+// (NV = j + 1 at compile time).  The earlier rotations of column j need only h and
+// h2, so a ninth warp of block 0 applies them while the others stream (a serial
+// chain of 2 j FP64 operations, 1.4 us at j = 28, that would otherwise follow the
+// norm); the last block adds the new rotation.
+constexpr int kNormThreads = kRedThreads + 32;
+
 template <int NV>
 __device__ __forceinline__ void orth_norm_body(const double *__restrict__ V, double *__restrict__ w, long n, int j,
                                                int m, double *partials, unsigned int *ticket, KrylovCtl *ctl,
                                                int selective, VBlk vb) {
-    const int nv = NV;
-    const bool re = need_reorth(ctl->h, nv, selective);   // else the first pass is subtracted here
+    constexpr int U = orth_unroll(NV);
+    const bool re = need_reorth(ctl->h, NV, selective);   // else the first pass is subtracted here
     __shared__ double hs[NVMAX];
-    for (int k = threadIdx.x; k < nv; k += blockDim.x) hs[k] = re ? ctl->h2[k] : ctl->h[k];
+    if (threadIdx.x < NV) hs[threadIdx.x] = re ? ctl->h2[threadIdx.x] : ctl->h[threadIdx.x];
     __syncthreads();
     double acc[1] = {0.0};
-    for (long i = vb.id * (long)blockDim.x + threadIdx.x; i < n; i += (long)vb.count * blockDim.x) {
-        double wi = w[i];
+    if (threadIdx.x < kRedThreads) {
+        const long st = (long)vb.count * kRedThreads;
+        long i = vb.id * (long)kRedThreads + threadIdx.x;
+        for (; i + (U - 1) * st < n; i += U * st) {
+            double wi[U], v[U][NV];
 #pragma unroll
-        for (int k = 0; k < NV; k++) wi -= hs[k] * V[k * n + i];
-        w[i] = wi;
-        acc[0] += wi * wi;
-    }
-    block_partials<1>(acc, 1, partials, vb);
-    if (last_block(ticket, vb.count)) {
-        __shared__ double nrm;
-        // the column and the earlier rotations, staged by the whole block so
-        // that thread 0's rotation chain reads shared memory only
+            for (int u = 0; u < U; u++) {
+                wi[u] = w[i + u * st];
+#pragma unroll
+                for (int k = 0; k < NV; k++) v[u][k] = V[k * n + i + u * st];
+            }
+#pragma unroll
+            for (int k = 0; k < NV; k++) {
+                const double hk = hs[k];
+#pragma unroll
+                for (int u = 0; u < U; u++) wi[u] -= hk * v[u][k];
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                w[i + u * st] = wi[u];
+                acc[0] += wi[u] * wi[u];
+            }
+        }
+        for (; i < n; i += st) {
+            double wi = w[i];
+#pragma unroll
+            for (int k = 0; k < NV; k++) wi -= hs[k] * V[k * n + i];
+            w[i] = wi;
+            acc[0] += wi * wi;
+        }
+    } else if (vb.id == 0) {
         __shared__ double col[NVMAX + 1], rcs[NVMAX + 1], rsn[NVMAX + 1];
-        for (int k = threadIdx.x; k <= j; k += blockDim.x) {
+        for (int k = threadIdx.x & 31; k <= j; k += 32) {
             col[k] = re ? ctl->h[k] + ctl->h2[k] : ctl->h[k];
             rcs[k] = ctl->cs[k];
             rsn[k] = ctl->sn[k];
         }
-        fold(partials, 1, &nrm, vb.count);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            *ticket = 0u;
-            const double hn = sqrt(nrm);
+        __syncwarp();
+        if (threadIdx.x == kRedThreads) {
             // two-product sums written as explicit FMAs: every kernel that
             // inlines this body (one system or a batch) rounds them alike
             for (int k = 0; k < j; k++) {
@@ -281,27 +369,40 @@ __device__ __forceinline__ void orth_norm_body(const double *__restrict__ V, dou
                 col[k] = fma(rcs[k], a, rsn[k] * c2);
                 col[k + 1] = fma(-rsn[k], a, rcs[k] * c2);
             }
-            const double a = col[j], bb = hn;
+        }
+        __syncwarp();
+        for (int k = threadIdx.x & 31; k <= j; k += 32) ctl->H[k * (SIM_MAX_M + 1) + j] = col[k];
+    }
+    block_partials<1>(acc, partials, vb);
+    if (last_block(ticket, vb.count)) {
+        __shared__ double nrm;
+        fold(partials, 1, &nrm, vb.count);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            *ticket = 0u;
+            const double hn = sqrt(nrm);
+            double *diag = ctl->H + j * (SIM_MAX_M + 1) + j;   // the rotated column's last entry, from block 0
+            const double a = __ldcg(diag), bb = hn;
             const double rr = sqrt(fma(a, a, bb * bb));
             double c, s;
             if (rr == 0.0) { c = 1.0; s = 0.0; }
             else { c = a / rr; s = bb / rr; }
             ctl->cs[j] = c; ctl->sn[j] = s;
-            col[j] = rr;
-            ctl->g[j + 1] = -s * ctl->g[j];
-            ctl->g[j] = c * ctl->g[j];
-            for (int k = 0; k <= j; k++) ctl->H[k * (SIM_MAX_M + 1) + j] = col[k];
+            *diag = rr;
+            const double gj = ctl->g[j], gn = -s * gj;
+            ctl->g[j + 1] = gn;
+            ctl->g[j] = c * gj;
             ctl->rnorm2 = hn;             // normaliser of v_{j+1}
             ctl->k = j + 1;
-            if (fabs(ctl->g[j + 1]) <= ctl->tol || j + 1 >= m) ctl->done = 1;
+            if (fabs(gn) <= ctl->tol || j + 1 >= m) ctl->done = 1;
         }
     }
 }
 
 template <int NV>
-__global__ void __launch_bounds__(SIM_THREADS, NV > 20 ? 2 : 3) orth_norm_kernel(const double *__restrict__ V, double *__restrict__ w,
-                                                                long n, int j, int m, double *partials,
-                                                                unsigned int *ticket, KrylovCtl *ctl, int selective) {
+__global__ void __launch_bounds__(kNormThreads, 2) orth_norm_kernel(const double *__restrict__ V, double *__restrict__ w,
+                                                                    long n, int j, int m, double *partials,
+                                                                    unsigned int *ticket, KrylovCtl *ctl, int selective) {
     if (ctl->done) return;
     orth_norm_body<NV>(V, w, n, j, m, partials, ticket, ctl, selective, grid_blk());
 }
@@ -321,30 +422,27 @@ __global__ void scale_kernel(const double *__restrict__ w, double *__restrict__ 
     scale_body(w, v, n, ctl, use_beta, grid_blk());
 }
 
-// y = H^{-1} g (k x k upper triangular), single thread
-// (H and g staged in shared memory by the block, so the one thread that runs
-// the dependent back substitution never waits on global memory)
+// y = H^{-1} g (k x k upper triangular) by one warp: lane r holds row r's right-hand
+// side, and each solved unknown is broadcast and subtracted from the rows above at
+// once (k dependent steps instead of k^2 / 2: 40 us -> 4 us at k = 30) (k <= 32)
 __device__ __forceinline__ void backsolve_body(KrylovCtl *ctl) {
     constexpr int LD = SIM_MAX_M + 1;
-    __shared__ double Hs[LD * LD], gs[LD], ys[LD];
-    const int k = ctl->k;
+    __shared__ double Hs[LD * LD];
+    const int k = ctl->k, lane = threadIdx.x & 31;
     for (int t = threadIdx.x; t < k * LD; t += blockDim.x) Hs[t] = ctl->H[t];
-    for (int t = threadIdx.x; t < k; t += blockDim.x) gs[t] = ctl->g[t];
+    double g0 = lane < k ? ctl->g[lane] : 0.0;
+    const double d0 = lane < k ? ctl->H[lane * LD + lane] : 1.0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = k - 1; i >= 0; i--) {
-            double t = gs[i];
-            for (int c = i + 1; c < k; c++) t -= Hs[i * LD + c] * ys[c];
-            ys[i] = t / Hs[i * LD + i];
-        }
+    for (int i = k - 1; i >= 0; i--) {
+        const double yi = __shfl_sync(0xffffffffu, g0 / d0, i);
+        if (lane == i) ctl->y[i] = yi;
+        else if (lane < i) g0 -= Hs[lane * LD + i] * yi;
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < k; t += blockDim.x) ctl->y[t] = ys[t];
 }
 
-__global__ void backsolve_kernel(KrylovCtl *ctl) { backsolve_body(ctl); }
+__global__ void __launch_bounds__(32) backsolve_kernel(KrylovCtl *ctl) { backsolve_body(ctl); }
 
-// x += sum_k y_k Z_k
+// x += sum_k y_k Z_k (six directions' loads in flight, added in order)
 template <typename Z>
 __device__ __forceinline__ void xupdate_body(double *__restrict__ x, const Z *__restrict__ Zb, long n,
                                              const KrylovCtl *ctl, VBlk vb) {
@@ -354,7 +452,15 @@ __device__ __forceinline__ void xupdate_body(double *__restrict__ x, const Z *__
     __syncthreads();
     for (long i = vb.id * (long)blockDim.x + threadIdx.x; i < n; i += (long)vb.count * blockDim.x) {
         double s = x[i];
-        for (int t = 0; t < k; t++) s += ys[t] * (double)Zb[t * n + i];
+        int t = 0;
+        for (; t + 6 <= k; t += 6) {
+            Z z[6];
+#pragma unroll
+            for (int u = 0; u < 6; u++) z[u] = Zb[(t + u) * n + i];
+#pragma unroll
+            for (int u = 0; u < 6; u++) s += ys[t + u] * (double)z[u];
+        }
+        for (; t < k; t++) s += ys[t] * (double)Zb[t * n + i];
         x[i] = s;
     }
 }
@@ -374,7 +480,7 @@ __device__ __forceinline__ bool resid_body(const double *__restrict__ b, const d
         r[i] = v;
         acc[0] += v * v;
     }
-    block_partials<1>(acc, 1, partials, vb);
+    block_partials<1>(acc, partials, vb);
     if (last_block(ticket, vb.count)) {
         __shared__ double nrm;
         fold(partials, 1, &nrm, vb.count);
@@ -385,7 +491,7 @@ __device__ __forceinline__ bool resid_body(const double *__restrict__ b, const d
     return false;
 }
 
-__global__ void __launch_bounds__(SIM_THREADS) resid_kernel(const double *__restrict__ b, const double *__restrict__ y,
+__global__ void __launch_bounds__(kRedThreads) resid_kernel(const double *__restrict__ b, const double *__restrict__ y,
                                                             double *__restrict__ r, long n, double *partials,
                                                             unsigned int *ticket, double *out) {
     resid_body(b, y, r, n, partials, ticket, out, grid_blk());
@@ -394,7 +500,7 @@ __global__ void __launch_bounds__(SIM_THREADS) resid_kernel(const double *__rest
 __global__ void norm_kernel(const double *__restrict__ v, long n, double *partials, unsigned int *ticket, double *out) {
     double acc[1] = {0.0};
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) acc[0] += v[i] * v[i];
-    block_partials<1>(acc, 1, partials);
+    block_partials<1>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double nrm;
         fold(partials, 1, &nrm);
@@ -417,7 +523,7 @@ __global__ void cycle_init_kernel(KrylovCtl *ctl) { cycle_init_body(ctl, 0); }
 // One launch covers every member: block b of the launch takes the work item
 // work[b] = (member, virtual block), finds the member's operands in the table
 // M and runs the single-system body on its share (the member's reductions
-// keep their own partials, ticket and virtual grid of SIM_RED_BLOCKS blocks,
+// keep their own partials, ticket and virtual grid of sim_red_blocks(n) blocks,
 // so each member's sums are the ones of a launch of its own).  A member whose
 // solve has converged (ctl->active = 0) or whose cycle is done returns at once.
 __device__ __forceinline__ const KMember &member_of(const KMember *M, const int2 *work, VBlk *vb, int count) {
@@ -426,14 +532,22 @@ __device__ __forceinline__ const KMember &member_of(const KMember *M, const int2
     vb->count = count;
     return M[wk.x];
 }
+// a block of the member's reduction grid (as wide as its own launches': nred)
+__device__ __forceinline__ const KMember &member_red(const KMember *M, const int2 *work, VBlk *vb) {
+    const int2 wk = work[blockIdx.x];
+    const KMember &m = M[wk.x];
+    vb->id = wk.y;
+    vb->count = m.nred;
+    return m;
+}
 
 __device__ __forceinline__ bool cycle_off(const KMember &m) { return *(volatile const int *)&m.ctl->done; }
 
 // start of a solve: r = b, x = 0, beta = ||b||, tol = theta ||b||, active
 // when beta is positive and finite
-__global__ void __launch_bounds__(SIM_THREADS) b_start_kernel(const KMember *M, const int2 *work) {
+__global__ void __launch_bounds__(kRedThreads) b_start_kernel(const KMember *M, const int2 *work) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (!m.rhs) return;                                  // not solving in this round
     double acc[1] = {0.0};
     for (long i = vb.id * (long)blockDim.x + threadIdx.x; i < m.n; i += (long)vb.count * blockDim.x) {
@@ -442,7 +556,7 @@ __global__ void __launch_bounds__(SIM_THREADS) b_start_kernel(const KMember *M, 
         m.x[i] = 0.0;
         acc[0] += v * v;
     }
-    block_partials<1>(acc, 1, m.red, vb);
+    block_partials<1>(acc, m.red, vb);
     if (last_block(m.ticket, vb.count)) {
         __shared__ double nrm;
         fold(m.red, 1, &nrm, vb.count);
@@ -468,7 +582,7 @@ __global__ void b_cycle_init_kernel(const KMember *M, const int2 *work) {
 // v_j = w / scale: j = 0 from the residual (use_beta), else from w
 __global__ void b_scale_kernel(const KMember *M, const int2 *work, int j, int use_beta) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (cycle_off(m)) return;
     scale_body(use_beta ? m.r : m.w, m.V + (size_t)j * m.n, m.n, m.ctl, use_beta, vb);
 }
@@ -486,26 +600,27 @@ __global__ void __launch_bounds__(512) b_spmv_kernel(const KMember *M, const int
 }
 
 template <int NV>
-__global__ void __launch_bounds__(SIM_THREADS, NV > 20 ? 2 : 3) b_dots_kernel(const KMember *M, const int2 *work) {
+__global__ void __launch_bounds__(kRedThreads, 2) b_dots_kernel(const KMember *M, const int2 *work) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (cycle_off(m)) return;
     dots_body<NV>(m.V, m.w, m.n, m.red, m.ticket, m.ctl->h, vb);
 }
 
 template <int NV>
-__global__ void __launch_bounds__(kOrthTile) b_orth_dots_kernel(const KMember *M, const int2 *work, int selective) {
+__global__ void __launch_bounds__(kRedThreads, NV > 17 ? 1 : 2) b_orth_dots_kernel(const KMember *M, const int2 *work,
+                                                                                  int selective) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, 2 * SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (cycle_off(m)) return;
     orth_dots_body<NV>(m.V, m.w, m.n, m.ctl->h, m.red, m.ticket, m.ctl->h2, selective, vb);
 }
 
 template <int NV>
-__global__ void __launch_bounds__(SIM_THREADS, NV > 20 ? 2 : 3) b_orth_norm_kernel(const KMember *M, const int2 *work,
-                                                                                  int mrestart, int selective) {
+__global__ void __launch_bounds__(kNormThreads, 2) b_orth_norm_kernel(const KMember *M, const int2 *work, int mrestart,
+                                                                     int selective) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (cycle_off(m)) return;
     orth_norm_body<NV>(m.V, m.w, m.n, NV - 1, mrestart, m.red, m.ticket, m.ctl, selective, vb);
 }
@@ -521,15 +636,15 @@ __global__ void b_backsolve_kernel(const KMember *M, const int2 *work) {
 template <typename Z>
 __global__ void b_xupdate_kernel(const KMember *M, const int2 *work) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (!(m.rhs && m.ctl->active)) return;
     xupdate_body<Z>(m.x, (const Z *)m.Z, m.n, m.ctl, vb);
 }
 
 // r = b - w, beta = ||r||; the member stays active while beta > tol (finite)
-__global__ void __launch_bounds__(SIM_THREADS) b_resid_kernel(const KMember *M, const int2 *work) {
+__global__ void __launch_bounds__(kRedThreads) b_resid_kernel(const KMember *M, const int2 *work) {
     VBlk vb;
-    const KMember &m = member_of(M, work, &vb, SIM_RED_BLOCKS);
+    const KMember &m = member_red(M, work, &vb);
     if (!(m.rhs && m.ctl->active)) return;
     if (resid_body(m.rhs, m.w, m.r, m.n, m.red, m.ticket, &m.ctl->beta, vb) && threadIdx.x == 0) {
         const double beta = m.ctl->beta;
@@ -543,32 +658,30 @@ template <int NV>
 struct OrthDispatch {
     static void dots(int nv, cudaStream_t st, const double *V, const double *w, long n, double *part, unsigned int *tk,
                      double *out, const int *done) {
-        if (nv == NV) dots_kernel<NV><<<SIM_RED_BLOCKS, SIM_THREADS, 0, st>>>(V, w, n, part, tk, out, done);
+        if (nv == NV) dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, part, tk, out, done);
         else OrthDispatch<NV - 1>::dots(nv, st, V, w, n, part, tk, out, done);
     }
     static void norm(int nv, cudaStream_t st, const double *V, double *w, long n, int m, double *part, unsigned int *tk,
                      KrylovCtl *ctl, int sel) {
-        if (nv == NV) orth_norm_kernel<NV><<<SIM_RED_BLOCKS, SIM_THREADS, 0, st>>>(V, w, n, NV - 1, m, part, tk, ctl, sel);
+        if (nv == NV) orth_norm_kernel<NV><<<sim_red_blocks(n), kNormThreads, 0, st>>>(V, w, n, NV - 1, m, part, tk, ctl, sel);
         else OrthDispatch<NV - 1>::norm(nv, st, V, w, n, m, part, tk, ctl, sel);
     }
     static void orth(int nv, cudaStream_t st, const double *V, double *w, long n, const double *h, double *part,
                      unsigned int *tk, double *out, const int *done, int sel) {
-        // 6 blocks of 128 threads per SM keep loads in flight while tiles are reduced
-        if (nv == NV) orth_dots_kernel<NV><<<2 * SIM_RED_BLOCKS, kOrthTile, 0, st>>>(V, w, n, h, part, tk, out, done, sel);
+        if (nv == NV) orth_dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, h, part, tk, out, done, sel);
         else OrthDispatch<NV - 1>::orth(nv, st, V, w, n, h, part, tk, out, done, sel);
     }
-    // batched: one launch per pass over every member (work lists of SIM_RED_BLOCKS
-    // and 2 SIM_RED_BLOCKS virtual blocks per member)
+    // batched: one launch per pass over every member's virtual blocks
     static void bdots(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred) {
-        if (nv == NV) b_dots_kernel<NV><<<nred, SIM_THREADS, 0, st>>>(M, wred);
+        if (nv == NV) b_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred);
         else OrthDispatch<NV - 1>::bdots(nv, st, M, wred, nred);
     }
-    static void borth(int nv, cudaStream_t st, const KMember *M, const int2 *worth, int north, int sel) {
-        if (nv == NV) b_orth_dots_kernel<NV><<<north, kOrthTile, 0, st>>>(M, worth, sel);
-        else OrthDispatch<NV - 1>::borth(nv, st, M, worth, north, sel);
+    static void borth(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int sel) {
+        if (nv == NV) b_orth_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred, sel);
+        else OrthDispatch<NV - 1>::borth(nv, st, M, wred, nred, sel);
     }
     static void bnorm(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int m, int sel) {
-        if (nv == NV) b_orth_norm_kernel<NV><<<nred, SIM_THREADS, 0, st>>>(M, wred, m, sel);
+        if (nv == NV) b_orth_norm_kernel<NV><<<nred, kNormThreads, 0, st>>>(M, wred, m, sel);
         else OrthDispatch<NV - 1>::bnorm(nv, st, M, wred, nred, m, sel);
     }
 };
@@ -593,7 +706,7 @@ struct OrthDispatch<0> {
 __device__ __forceinline__ bool bdone(const BicgCtl *c) { return *(volatile const int *)&c->done; }
 
 // start or restart from the current residual: rh = r, rho = (r, r)
-__global__ void __launch_bounds__(SIM_THREADS) bicg_restart_kernel(const double *__restrict__ r, double *__restrict__ rh,
+__global__ void __launch_bounds__(kRedThreads) bicg_restart_kernel(const double *__restrict__ r, double *__restrict__ rh,
                                                                    long n, double *partials, unsigned int *ticket,
                                                                    BicgCtl *ctl) {
     double acc[1] = {0.0};
@@ -602,7 +715,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_restart_kernel(const double 
         rh[i] = v;
         acc[0] += v * v;
     }
-    block_partials<1>(acc, 1, partials);
+    block_partials<1>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double d;
         fold(partials, 1, &d);
@@ -638,13 +751,13 @@ __global__ void bicg_p_kernel(const double *__restrict__ r, const double *__rest
 }
 
 // alpha = rho / (rh, v); one iteration counted
-__global__ void __launch_bounds__(SIM_THREADS) bicg_alpha_kernel(const double *__restrict__ rh, const double *__restrict__ v,
+__global__ void __launch_bounds__(kRedThreads) bicg_alpha_kernel(const double *__restrict__ rh, const double *__restrict__ v,
                                                                  long n, double *partials, unsigned int *ticket,
                                                                  BicgCtl *ctl) {
     if (bdone(ctl)) return;
     double acc[1] = {0.0};
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) acc[0] += rh[i] * v[i];
-    block_partials<1>(acc, 1, partials);
+    block_partials<1>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double d;
         fold(partials, 1, &d);
@@ -659,7 +772,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_alpha_kernel(const double *_
 }
 
 // s = r - alpha v; ||s|| <= tol ends the iteration at its half step (iteration j of the chunk)
-__global__ void __launch_bounds__(SIM_THREADS) bicg_s_kernel(const double *__restrict__ r, const double *__restrict__ v,
+__global__ void __launch_bounds__(kRedThreads) bicg_s_kernel(const double *__restrict__ r, const double *__restrict__ v,
                                                              double *__restrict__ sv, long n, double *partials,
                                                              unsigned int *ticket, BicgCtl *ctl, int j) {
     if (bdone(ctl)) return;
@@ -670,7 +783,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_s_kernel(const double *__res
         sv[i] = t;
         acc[0] += t * t;
     }
-    block_partials<1>(acc, 1, partials);
+    block_partials<1>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double d;
         fold(partials, 1, &d);
@@ -692,7 +805,7 @@ __global__ void bicg_xhalf_kernel(double *__restrict__ x, const Z *__restrict__ 
 }
 
 // omega = (t, s) / (t, t)
-__global__ void __launch_bounds__(SIM_THREADS) bicg_omega_kernel(const double *__restrict__ t, const double *__restrict__ sv,
+__global__ void __launch_bounds__(kRedThreads) bicg_omega_kernel(const double *__restrict__ t, const double *__restrict__ sv,
                                                                  long n, double *partials, unsigned int *ticket,
                                                                  BicgCtl *ctl) {
     if (bdone(ctl)) return;
@@ -702,7 +815,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_omega_kernel(const double *_
         acc[0] += ti * ti;
         acc[1] += ti * sv[i];
     }
-    block_partials<2>(acc, 2, partials);
+    block_partials<2>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double d[2];
         fold(partials, 2, d);
@@ -716,7 +829,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_omega_kernel(const double *_
 
 // x += alpha p^ + omega s^; r = s - omega t; rho for the next iteration; tests
 template <typename Z>
-__global__ void __launch_bounds__(SIM_THREADS) bicg_xr_kernel(double *__restrict__ x, const Z *__restrict__ ph,
+__global__ void __launch_bounds__(kRedThreads) bicg_xr_kernel(double *__restrict__ x, const Z *__restrict__ ph,
                                                               const Z *__restrict__ sh, const double *__restrict__ sv,
                                                               const double *__restrict__ t, double *__restrict__ r,
                                                               const double *__restrict__ rh, long n, double *partials,
@@ -731,7 +844,7 @@ __global__ void __launch_bounds__(SIM_THREADS) bicg_xr_kernel(double *__restrict
         acc[0] += rh[i] * ri;
         acc[1] += ri * ri;
     }
-    block_partials<2>(acc, 2, partials);
+    block_partials<2>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double d[2];
         fold(partials, 2, d);
@@ -758,7 +871,7 @@ __global__ void diff_norm_kernel(const double *__restrict__ a, const double *__r
         const double d = a[i] - b[i];
         acc[0] += d * d;
     }
-    block_partials<1>(acc, 1, partials);
+    block_partials<1>(acc, partials);
     if (last_block(ticket)) {
         __shared__ double nrm;
         fold(partials, 1, &nrm);
@@ -798,7 +911,7 @@ static sim_status spmv_done(sim_t *s, const void *x, bool xf, double *y, const i
 sim_status k_spmv_f(sim_t *s, const float *x, double *y) { return spmv_done(s, x, true, y, nullptr); }
 
 sim_status k_norm2(sim_t *s, const double *v, long n, double *out) {
-    norm_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(v, n, s->red, s->ticket, s->scal);
+    norm_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(v, n, s->red, s->ticket, s->scal);
     SIM_LAUNCHED(s);
     SIM_CK(s, cudaMemcpyAsync(s->h_pinned, s->scal, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     SIM_CK(s, cudaStreamSynchronize(s->stream));
@@ -817,7 +930,7 @@ static sim_status enqueue_cycle(sim_t *s) {
     const int *done = &ctl->done;
     cycle_init_kernel<<<1, 64, 0, s->stream>>>(ctl);
     SIM_LAUNCHED(s);
-    scale_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->r, s->V, n, ctl, 1);
+    scale_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->r, s->V, n, ctl, 1);
     SIM_LAUNCHED(s);
     for (int j = 0; j < m; j++) {
         double *vj = s->V + (size_t)j * n;
@@ -831,7 +944,7 @@ static sim_status enqueue_cycle(sim_t *s) {
         SIM_LAUNCHED(s);
         OrthDispatch<SIM_MAX_M>::norm(j + 1, s->stream, s->V, s->w, n, m, s->red, s->ticket, ctl, s->opt.orth);
         SIM_LAUNCHED(s);
-        scale_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->w, s->V + (size_t)(j + 1) * n, n, ctl, 0);
+        scale_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->w, s->V + (size_t)(j + 1) * n, n, ctl, 0);
         SIM_LAUNCHED(s);
     }
     return SIM_OK;
@@ -851,7 +964,7 @@ sim_status k_orth_step(sim_t *s, int nv) {
     SIM_LAUNCHED(s);
     OrthDispatch<SIM_MAX_M>::norm(nv, s->stream, s->V, s->w, n, s->m, s->red, s->ticket, ctl, s->opt.orth);
     SIM_LAUNCHED(s);
-    scale_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->w, s->V + (size_t)nv * n, n, ctl, 0);
+    scale_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->w, s->V + (size_t)nv * n, n, ctl, 0);
     SIM_LAUNCHED(s);
     return SIM_OK;
 }
@@ -917,11 +1030,11 @@ sim_status k_fgmres(sim_t *s, const double *b, double *x, sim_linear_info *info)
         }
         backsolve_kernel<<<1, 32, 0, s->stream>>>(ctl);
         SIM_LAUNCHED(s);
-        if (zf) xupdate_kernel<float><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const float *)s->Z, n, ctl);
-        else xupdate_kernel<double><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const double *)s->Z, n, ctl);
+        if (zf) xupdate_kernel<float><<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(x, (const float *)s->Z, n, ctl);
+        else xupdate_kernel<double><<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(x, (const double *)s->Z, n, ctl);
         SIM_LAUNCHED(s);
         if (k_spmv(s, x, s->w) != SIM_OK) return s->err;
-        resid_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(b, s->w, s->r, n, s->red, s->ticket, &ctl->beta);
+        resid_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(b, s->w, s->r, n, s->red, s->ticket, &ctl->beta);
         SIM_LAUNCHED(s);
         SIM_CK(s, cudaMemcpyAsync(s->ctl_host, ctl, offsetof(KrylovCtl, h), cudaMemcpyDeviceToHost, s->stream));
         SIM_CK(s, cudaStreamSynchronize(s->stream));
@@ -972,26 +1085,26 @@ static sim_status enqueue_bicg_chunk(sim_t *s, double *x) {
     bicg_chunk_init_kernel<<<1, 1, 0, s->stream>>>(ctl);
     SIM_LAUNCHED(s);
     for (int j = 0; j < kBicgChunk; j++) {
-        bicg_p_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->r, v, p, n, ctl);
+        bicg_p_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->r, v, p, n, ctl);
         SIM_LAUNCHED(s);
         if (cpr_apply(s, p, ph, done) != SIM_OK) return s->err;
         if (spmv_done(s, ph, zf, v, done) != SIM_OK) return s->err;
-        bicg_alpha_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(rh, v, n, s->red, s->ticket, ctl);
+        bicg_alpha_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(rh, v, n, s->red, s->ticket, ctl);
         SIM_LAUNCHED(s);
-        bicg_s_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->r, v, sv, n, s->red, s->ticket, ctl, j);
+        bicg_s_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(s->r, v, sv, n, s->red, s->ticket, ctl, j);
         SIM_LAUNCHED(s);
-        if (zf) bicg_xhalf_kernel<float><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const float *)ph, n, ctl, j);
-        else bicg_xhalf_kernel<double><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const double *)ph, n, ctl, j);
+        if (zf) bicg_xhalf_kernel<float><<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(x, (const float *)ph, n, ctl, j);
+        else bicg_xhalf_kernel<double><<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(x, (const double *)ph, n, ctl, j);
         SIM_LAUNCHED(s);
         if (cpr_apply(s, sv, sh, done) != SIM_OK) return s->err;
         if (spmv_done(s, sh, zf, t, done) != SIM_OK) return s->err;
-        bicg_omega_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(t, sv, n, s->red, s->ticket, ctl);
+        bicg_omega_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(t, sv, n, s->red, s->ticket, ctl);
         SIM_LAUNCHED(s);
         if (zf)
-            bicg_xr_kernel<float><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const float *)ph, (const float *)sh, sv, t,
+            bicg_xr_kernel<float><<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(x, (const float *)ph, (const float *)sh, sv, t,
                                                                                 s->r, rh, n, s->red, s->ticket, ctl);
         else
-            bicg_xr_kernel<double><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(x, (const double *)ph, (const double *)sh,
+            bicg_xr_kernel<double><<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(x, (const double *)ph, (const double *)sh,
                                                                                  sv, t, s->r, rh, n, s->red, s->ticket, ctl);
         SIM_LAUNCHED(s);
     }
@@ -1036,7 +1149,7 @@ static sim_status launch_bicg_chunk(sim_t *s, double *x) {
 static sim_status bicg_true_residual(sim_t *s, const double *b, const double *x) {
     const long n = (long)s->N * s->b;
     if (k_spmv(s, x, s->w) != SIM_OK) return s->err;
-    resid_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(b, s->w, s->r, n, s->red, s->ticket, &s->bctl->rnorm);
+    resid_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(b, s->w, s->r, n, s->red, s->ticket, &s->bctl->rnorm);
     SIM_LAUNCHED(s);
     SIM_CK(s, cudaMemcpyAsync(s->bctl_host, s->bctl, sizeof(BicgCtl), cudaMemcpyDeviceToHost, s->stream));
     SIM_CK(s, cudaStreamSynchronize(s->stream));
@@ -1063,7 +1176,7 @@ sim_status k_bicgstab(sim_t *s, const double *b, double *x, sim_linear_info *inf
     BicgCtl *ctl = s->bctl;
     bicg_init_kernel<<<1, 1, 0, s->stream>>>(ctl, tol, s->opt.lin_max_iter);
     SIM_LAUNCHED(s);
-    bicg_restart_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->r, s->V, n, s->red, s->ticket, ctl);
+    bicg_restart_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(s->r, s->V, n, s->red, s->ticket, ctl);
     SIM_LAUNCHED(s);
     for (;;) {
         if (launch_bicg_chunk(s, x) != SIM_OK) return s->err;
@@ -1076,7 +1189,7 @@ sim_status k_bicgstab(sim_t *s, const double *b, double *x, sim_linear_info *inf
         li.r_norm = h.rnorm;
         if (h.rnorm <= tol) { li.converged = 1; break; }
         if (!(h.rnorm == h.rnorm) || h.it >= h.max_it) break;
-        bicg_restart_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(s->r, s->V, n, s->red, s->ticket, ctl);
+        bicg_restart_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(s->r, s->V, n, s->red, s->ticket, ctl);
         SIM_LAUNCHED(s);
         li.restarts++;
     }
@@ -1091,7 +1204,7 @@ sim_status k_linear_solve(sim_t *s, const double *b, double *x, sim_linear_info 
 }
 
 sim_status k_diff_norm2(sim_t *s, const double *a, const double *b, long n, double *out) {
-    diff_norm_kernel<<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(a, b, n, s->red, s->ticket, s->scal);
+    diff_norm_kernel<<<sim_red_blocks(n), kRedThreads, 0, s->stream>>>(a, b, n, s->red, s->ticket, s->scal);
     SIM_LAUNCHED(s);
     SIM_CK(s, cudaMemcpyAsync(s->h_pinned, s->scal, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     SIM_CK(s, cudaStreamSynchronize(s->stream));
@@ -1122,8 +1235,8 @@ struct KrylovBatch {
     KMember *dmem = nullptr; size_t mem_cap = 0;
     int2 *dwork = nullptr; size_t work_cap = 0;
     double *dout = nullptr, *hout = nullptr; int out_cap = 0;
-    long red_off = 0, orth_off = 0, one_off = 0, cell_off = 0;
-    int red_n = 0, orth_n = 0, one_n = 0, cell_n = 0;
+    long red_off = 0, one_off = 0, cell_off = 0;
+    int red_n = 0, one_n = 0, cell_n = 0;
     CprBatch *cpr = nullptr;
     cudaGraphExec_t exec = nullptr;
     int64_t nodes = 0, launches = 0;
@@ -1163,7 +1276,7 @@ static cudaError_t enqueue_batch_cycle(KrylovBatch *kb, cudaStream_t st, int64_t
     const int2 *W = kb->dwork;
     int64_t n = 0;
     b_cycle_init_kernel<<<kb->one_n, 64, 0, st>>>(M, W + kb->one_off); n++;
-    b_scale_kernel<<<kb->red_n, SIM_THREADS, 0, st>>>(M, W + kb->red_off, 0, 1); n++;
+    b_scale_kernel<<<kb->red_n, kRedThreads, 0, st>>>(M, W + kb->red_off, 0, 1); n++;
     for (int j = 0; j < kb->m; j++) {
         const int a = cpr_batch_apply(kb->cpr, st, j);
         if (a < 0) return cudaErrorLaunchFailure;
@@ -1176,9 +1289,9 @@ static cudaError_t enqueue_batch_cycle(KrylovBatch *kb, cudaStream_t st, int64_t
             else b_spmv_kernel<3, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(M, W + kb->cell_off, j, 0);
         }
         OrthDispatch<SIM_MAX_M>::bdots(j + 1, st, M, W + kb->red_off, kb->red_n);
-        OrthDispatch<SIM_MAX_M>::borth(j + 1, st, M, W + kb->orth_off, kb->orth_n, kb->orth);
+        OrthDispatch<SIM_MAX_M>::borth(j + 1, st, M, W + kb->red_off, kb->red_n, kb->orth);
         OrthDispatch<SIM_MAX_M>::bnorm(j + 1, st, M, W + kb->red_off, kb->red_n, kb->m, kb->orth);
-        b_scale_kernel<<<kb->red_n, SIM_THREADS, 0, st>>>(M, W + kb->red_off, j + 1, 0);
+        b_scale_kernel<<<kb->red_n, kRedThreads, 0, st>>>(M, W + kb->red_off, j + 1, 0);
         n += 5;
     }
     *launches = n;
@@ -1200,10 +1313,10 @@ sim_status k_fgmres_batch(KrylovBatch *kb, sim_t *const *ms, int nm, cudaStream_
     kb->nm = nm; kb->m = s0->m; kb->b = s0->b; kb->zf = sim_mixed(s0) ? 1 : 0; kb->orth = s0->opt.orth;
     std::vector<KMember> hm(nm);
     std::vector<int2> work;
-    auto add = [&](long *off, int *count, int per_member_fixed, bool cells) {
+    auto add = [&](long *off, int *count, auto blocks_of) {
         *off = (long)work.size();
         for (int k = 0; k < nm; k++) {
-            const int nb = cells ? sim_blocks(ms[k]->N, SIM_THREADS) : per_member_fixed;
+            const int nb = blocks_of(k);
             for (int q = 0; q < nb; q++) work.push_back(make_int2(k, q));
         }
         *count = (int)((long)work.size() - *off);
@@ -1213,12 +1326,11 @@ sim_status k_fgmres_batch(KrylovBatch *kb, sim_t *const *ms, int nm, cudaStream_
         KMember &m = hm[k];
         m.g = s->gd; m.n = (long)s->N * s->b; m.theta = s->theta; m.J = s->J;
         m.V = s->V; m.w = s->w; m.r = s->r; m.x = s->dx; m.rhs = s->bl; m.Z = s->Z;
-        m.ctl = s->ctl; m.red = s->red; m.ticket = s->ticket;
+        m.ctl = s->ctl; m.red = s->red; m.ticket = s->ticket; m.nred = sim_red_blocks(m.n);
     }
-    add(&kb->red_off, &kb->red_n, SIM_RED_BLOCKS, false);
-    add(&kb->orth_off, &kb->orth_n, 2 * SIM_RED_BLOCKS, false);
-    add(&kb->one_off, &kb->one_n, 1, false);
-    add(&kb->cell_off, &kb->cell_n, 0, true);
+    add(&kb->red_off, &kb->red_n, [&](int k) { return hm[k].nred; });
+    add(&kb->one_off, &kb->one_n, [&](int) { return 1; });
+    add(&kb->cell_off, &kb->cell_n, [&](int k) { return sim_blocks(ms[k]->N, SIM_THREADS); });
     cudaError_t e;
     if ((e = kgrow((void **)&kb->dmem, &kb->mem_cap, sizeof(KMember) * nm)) != cudaSuccess) return fail("allocation", e);
     if ((e = kgrow((void **)&kb->dwork, &kb->work_cap, sizeof(int2) * work.size())) != cudaSuccess) return fail("allocation", e);
@@ -1235,7 +1347,7 @@ sim_status k_fgmres_batch(KrylovBatch *kb, sim_t *const *ms, int nm, cudaStream_
         return fail("table upload", e);
     if ((e = cpr_batch_build(kb->cpr, ms, nm, st)) != cudaSuccess) return fail("CPR tables", e);   // synchronises st
     // start: r = b, x = 0, beta = ||b||, tolerance, active
-    b_start_kernel<<<kb->red_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
+    b_start_kernel<<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
     kb->launches++;
     b_gather_kernel<<<kb->one_n, 32, 0, st>>>(kb->dmem, kb->dwork + kb->one_off, kb->dout);
     kb->launches++;
@@ -1281,11 +1393,11 @@ sim_status k_fgmres_batch(KrylovBatch *kb, sim_t *const *ms, int nm, cudaStream_
         if ((e = cudaGraphLaunch(kb->exec, st)) != cudaSuccess) return fail("cycle", e);
         kb->launches += kb->nodes;
         b_backsolve_kernel<<<kb->one_n, 32, 0, st>>>(kb->dmem, kb->dwork + kb->one_off);
-        if (kb->zf) b_xupdate_kernel<float><<<kb->red_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
-        else b_xupdate_kernel<double><<<kb->red_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
+        if (kb->zf) b_xupdate_kernel<float><<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
+        else b_xupdate_kernel<double><<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
         if (kb->b == 2) b_spmv_kernel<2, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->cell_off, 0, 1);
         else b_spmv_kernel<3, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->cell_off, 0, 1);
-        b_resid_kernel<<<kb->red_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
+        b_resid_kernel<<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
         b_gather_kernel<<<kb->one_n, 32, 0, st>>>(kb->dmem, kb->dwork + kb->one_off, kb->dout);
         kb->launches += 5;
         if ((e = cudaGetLastError()) != cudaSuccess) return fail("launch", e);

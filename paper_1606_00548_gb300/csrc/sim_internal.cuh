@@ -23,8 +23,26 @@ struct NvtxRange {
 #define SIM_MAX_PVT 64
 #define SIM_MAX_M 32
 #define SIM_MAX_ELL 512      // widest coarse AMG row: a wider Galerkin row stops coarsening
-#define SIM_RED_BLOCKS 456   // 3 x 152 SMs: grid of the reduction kernels (one wave at <= 85 registers)
+#define SIM_RED_BLOCKS 456   // 3 x 152 SMs: grid of the state's reductions (CNV, masses, finiteness)
 #define SIM_THREADS 256
+
+// Reductions of the Krylov solvers over n entries: threads of a block that stream
+// and the blocks of the grid.  One block per SM: the kernels are bound by the FP64
+// pipe, which 8 warps keep busy, and every further block adds its own reduction and
+// 8 bytes a value for the last block to fold (600k entries, 16 vectors: dots 27 us,
+// update-and-dots 42 us; with two blocks per SM 31 and 46, with three 34 and 52).
+// From 2M entries the loads in flight count more than that (12M entries, 16 vectors:
+// dots 376 us, norm 347 us with two blocks per SM, 433 and 445 with one).
+constexpr int kRedThreads = 256;
+inline int sim_red_blocks(long n) {
+    const long want = (n + kRedThreads - 1) / kRedThreads, most = n >= (1L << 21) ? 304 : 152;
+    return (int)(want < 1 ? 1 : want < most ? want : most);
+}
+// blocks of SIM_THREADS of an elementwise pass over n entries: up to one full wave
+inline int sim_stream_blocks(long n) {
+    const long want = (n + SIM_THREADS - 1) / SIM_THREADS;
+    return (int)(want < 1 ? 1 : want < 1216 ? want : 1216);
+}
 
 // fluid and rock constants, passed by value as a kernel parameter (about
 // 3.3 KB, under the 4 KB parameter limit), so handles never share state
@@ -72,6 +90,7 @@ struct KMember {
     KrylovCtl *ctl;
     double *red;             // the member's reduction partials and ticket
     unsigned int *ticket;
+    int nred;                // virtual blocks of its reductions (sim_red_blocks(n))
 };
 
 // BiCGSTAB scalars (device); flag: 1 recursive residual met the tolerance,
@@ -146,7 +165,7 @@ struct sim {
     double cum_well[3] = {0, 0, 0};
 
     // reductions
-    double *red = nullptr;       // partial sums [SIM_MAX_M+2][SIM_RED_BLOCKS]
+    double *red = nullptr;       // partial sums [SIM_MAX_M+2][blocks of the reduction]
     double *scal = nullptr;      // small device scalars
     unsigned int *ticket = nullptr;
     double *h_pinned = nullptr;  // pinned host mirror for small reads
