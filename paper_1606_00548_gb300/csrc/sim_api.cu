@@ -216,14 +216,21 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     FluidConst &c = s->fc;
     memset(&c, 0, sizeof(c));
     c.model = f->model; c.b = s->b; c.npvt = f->model == 3 ? f->npvt : 0;
-    c.rho_w_ref = f->rho_w_ref; c.rho_o_ref = f->rho_o_ref; c.c_w = f->c_w; c.c_o = f->c_o; c.mu_w = f->mu_w; c.mu_o = f->mu_o;
+    c.rho_w_ref = f->rho_w_ref; c.rho_o_ref = f->rho_o_ref; c.c_w = f->c_w; c.c_o = f->c_o;
     c.rho_ws = f->rho_ws; c.rho_os = f->rho_os; c.rho_gs = f->rho_gs; c.bw_c = f->bw_c; c.bw_pref = f->bw_pref;
     c.bo_c_us = f->bo_c_us; c.muo_c_us = f->muo_c_us;
     c.swc = f->swc; c.sor = f->sor; c.sgc = f->sgc; c.sorg = f->sorg; c.nw = f->nw; c.now = f->now; c.ng = f->ng; c.nog = f->nog;
     c.c_rock = r->c_rock; c.p_ref = r->p_ref;
-    for (int k = 0; k < c.npvt; k++) {
-        c.pvt_p[k] = f->pvt_p[k]; c.pvt_bo[k] = f->pvt_bo[k]; c.pvt_rs[k] = f->pvt_rs[k];
-        c.pvt_muo[k] = f->pvt_muo[k]; c.pvt_bg[k] = f->pvt_bg[k]; c.pvt_mug[k] = f->pvt_mug[k];
+    c.i_muw = 1.0 / f->mu_w; c.i_muo = 1.0 / f->mu_o; c.i_mob = 1.0 / (1.0 - f->swc - f->sor);
+    c.i_mobg = 1.0 / (1.0 - f->swc - f->sorg - f->sgc); c.i_mobog = 1.0 / (1.0 - f->swc - f->sorg);
+    std::vector<double> pvt;                 // interval rows: p, then value and slope per column
+    for (int k = 0; k + 1 < c.npvt; k++) {
+        const double *col[5] = {f->pvt_bo, f->pvt_rs, f->pvt_muo, f->pvt_bg, f->pvt_mug};
+        pvt.push_back(f->pvt_p[k]);
+        for (const double *v : col) {
+            pvt.push_back(v[k]);
+            pvt.push_back((v[k + 1] - v[k]) / (f->pvt_p[k + 1] - f->pvt_p[k]));
+        }
     }
     for (int k = 0; k < 3; k++) c.cnv_rho[k] = f->cnv_rho[k] > 0 ? f->cnv_rho[k] : 1.0;
 
@@ -239,7 +246,6 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     const long n = N * b;
     const bool mixed = o->precision == SIM_PRECISION_MIXED;
     const size_t tsz = mixed ? sizeof(float) : sizeof(double);
-    const int nq = b == 2 ? 4 : 7;
     bool ok = true;
     auto A = [&](size_t bytes) -> void * { void *p = ok ? sim_alloc(s, bytes) : nullptr; if (!p) ok = false; return p; };
     s->T = (double *)A(sizeof(double) * 3 * N);
@@ -274,7 +280,9 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     s->mold = (double *)A(sizeof(double) * n);
     s->R = (double *)A(sizeof(double) * n);
     s->J = (double *)A(sizeof(double) * 7 * b * b * N);
-    s->props = (double *)A(sizeof(double) * nq * (b + 1) * N);
+    s->props = (double *)A(sizeof(double) * (b == 2 ? 10 : 21) * N);
+    double *pvt_dev = (double *)A(sizeof(double) * (pvt.size() + 1));
+    c.pvt = pvt_dev;
     s->qtot = (double *)A(sizeof(double) * 4);
     s->red = (double *)A(sizeof(double) * (SIM_MAX_M + 2) * SIM_RED_BLOCKS);
     s->scal = (double *)A(sizeof(double) * 64);
@@ -350,6 +358,11 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     cudaMemsetAsync(s->ticket, 0, sizeof(unsigned int) * 4, s->stream);
     cudaMemsetAsync(s->x, 0, sizeof(double) * n, s->stream);
     cudaMemsetAsync(s->ph, 1, N, s->stream);
+    if (!pvt.empty() &&
+        cudaMemcpy(pvt_dev, pvt.data(), sizeof(double) * pvt.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+        sim_destroy(s);
+        return sim_fail(nullptr, SIM_ECUDA, "PVT table upload failed");
+    }
     if (ok && nwells > 0) {
         std::vector<int> cp;
         if (nrate > 0) {

@@ -44,16 +44,20 @@ inline int sim_stream_blocks(long n) {
     return (int)(want < 1 ? 1 : want < 1216 ? want : 1216);
 }
 
-// fluid and rock constants, passed by value as a kernel parameter (about
-// 3.3 KB, under the 4 KB parameter limit), so handles never share state
+// fluid and rock constants, passed by value as a kernel parameter, so handles never
+// share state; the PVT table is the handle's device array of npvt - 1 interval rows
+// (p, then value and slope of Bo, Rs, mu_o, Bg, mu_g), its slopes divided once on
+// the host
+constexpr int SIM_PVT_ROW = 11;
 struct FluidConst {
     int model, b, npvt;
-    double rho_w_ref, rho_o_ref, c_w, c_o, mu_w, mu_o;
+    double rho_w_ref, rho_o_ref, c_w, c_o;
     double rho_ws, rho_os, rho_gs, bw_c, bw_pref, bo_c_us, muo_c_us;
     double swc, sor, sgc, sorg, nw, now, ng, nog;
     double c_rock, p_ref;
-    double pvt_p[SIM_MAX_PVT], pvt_bo[SIM_MAX_PVT], pvt_rs[SIM_MAX_PVT], pvt_muo[SIM_MAX_PVT],
-        pvt_bg[SIM_MAX_PVT], pvt_mug[SIM_MAX_PVT];
+    // reciprocals: 1 / mu_w, 1 / mu_o, 1 / (1 - swc - sor), 1 / (1 - swc - sorg - sgc), 1 / (1 - swc - sorg)
+    double i_muw, i_muo, i_mob, i_mobg, i_mobog;
+    const double *pvt;
     double cnv_rho[3];
 };
 
@@ -160,7 +164,7 @@ struct sim {
     int8_t *ph = nullptr, *ph_old = nullptr;
     double *mold = nullptr;                  // [b][N]
     double *R = nullptr, *J = nullptr;       // [b][N], [7][b][b][N]
-    double *props = nullptr;                 // [nq*4][N]
+    double *props = nullptr;                 // [10 (b = 2) or 21][N] densities and mobilities (assemble.cu)
     double *qtot = nullptr;                  // [3] well rates of the last assembly
     double cum_well[3] = {0, 0, 0};
 
