@@ -317,18 +317,19 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
         s->x0 = A(tsz * n);
     }
     s->partner = (int *)A(sizeof(int) * N);
-    s->pick = (int *)A(sizeof(int) * (N + 1));   // also holds founder ids + total
+    s->pick = (int *)A(sizeof(int) * N);
+    s->pick2 = (int *)A(sizeof(int) * N);
+    s->absorbed = (int *)A(sizeof(int) * 6 * N);
     s->aggA = (int *)A(sizeof(int) * N);
     s->aggB = (int *)A(sizeof(int) * N);
     s->host = (int *)A(sizeof(int) * N);
-    s->flag = (int *)A(sizeof(int) * N);
-    s->cnt = (int *)A(sizeof(int) * (N + 1));
+    s->cnt = (int *)A(sizeof(int) * N);
     s->moffA = (int *)A(sizeof(int) * (N + 1));
     s->memA = (int *)A(sizeof(int) * N);
     s->moffB = (int *)A(sizeof(int) * (N + 1));
     s->memB = (int *)A(sizeof(int) * N);
-    s->scan = (int *)A(sizeof(int) * (N / 4096 + 2));
-    s->iscal = (int *)A(sizeof(int) * 8);
+    s->scan = (int *)A(sizeof(int) * 3 * (N / 1024 + 2));
+    s->iscal = (int *)A(sizeof(int) * 16);
     if (!ok) {
         std::string m = s->msg;
         sim_destroy(s);

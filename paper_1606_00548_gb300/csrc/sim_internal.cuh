@@ -116,6 +116,7 @@ struct AmgLevel {
     int *moff = nullptr, *mem = nullptr;   // members of each next-level aggregate, ascending (CSR)
     void *f = nullptr, *e = nullptr, *e2 = nullptr;   // V-cycle vectors (apply precision)
     void *coarse_inv = nullptr;  // coarsest: dense inverse, row-major n*n (FP64 in both forms)
+    void *work = nullptr;        // the allocation dinvT, f, e, e2, colA and an FP32 valT lie in
 };
 
 struct sim {
@@ -223,11 +224,9 @@ struct sim {
     void *rhT = nullptr, *x0 = nullptr;   // [b][N] CPR-FPF: L r - Ahat x0 and the first stage-F result
     std::vector<AmgLevel> lev;
     // AMG setup scratch
-    int *partner = nullptr, *pick = nullptr, *host = nullptr, *flag = nullptr, *cnt = nullptr;
+    int *partner = nullptr, *pick = nullptr, *pick2 = nullptr, *host = nullptr, *cnt = nullptr, *absorbed = nullptr;
     int *aggA = nullptr, *moffA = nullptr, *memA = nullptr, *aggB = nullptr, *moffB = nullptr, *memB = nullptr;
     int *scan = nullptr, *iscal = nullptr;
-    int *tcol = nullptr; double *tval = nullptr;   // intermediate (pass-1) matrix
-    int tcap = 0;
 };
 
 // ---- error helpers --------------------------------------------------------
