@@ -616,7 +616,8 @@ __device__ __forceinline__ void each_member(const AggPass &P, const Mat<double> 
     }
 }
 
-constexpr int kAggPer = 4;       // nodes per thread: a chunk is kAggPer * blockDim.x nodes
+// a chunk is one block's nodes, one per thread (four per thread in turn made the
+// second pass's launch 65 us at 85k nodes: a founder's lists are a chain of loads)
 __device__ __forceinline__ void agg_counts(const AggPass &P, const Mat<double> &A, int i, int (&c)[3]) {
     c[0] = c[1] = c[2] = 0;
     int p;
@@ -639,13 +640,8 @@ __device__ __forceinline__ int block_sum(int v) {
 
 __global__ void agg_sizes_kernel(AggPass P, Mat<double> A) {
     if (unfinished(A)) return;
-    int t[3] = {0, 0, 0};
-    const int base = blockIdx.x * blockDim.x * kAggPer;
-    for (int u = 0; u < kAggPer; u++) {
-        int c[3];
-        agg_counts(P, A, base + u * blockDim.x + threadIdx.x, c);
-        for (int q = 0; q < 3; q++) t[q] += c[q];
-    }
+    int t[3];
+    agg_counts(P, A, blockIdx.x * blockDim.x + threadIdx.x, t);
     for (int q = 0; q < 3; q++) {
         const int v = block_sum(t[q]);
         if (threadIdx.x == 0) P.csum[q * gridDim.x + blockIdx.x] = v;
@@ -668,13 +664,9 @@ __global__ void agg_write_kernel(AggPass P, Mat<double> A) {
     if (unfinished(A)) return;
     constexpr int kLocal = 24;
     __shared__ int wsum[3][32];
-    const int base_i = (blockIdx.x * blockDim.x + threadIdx.x) * kAggPer, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int c[kAggPer][3], t[3] = {0, 0, 0}, pre[3];
-#pragma unroll
-    for (int u = 0; u < kAggPer; u++) {
-        agg_counts(P, A, base_i + u, c[u]);
-        for (int q = 0; q < 3; q++) t[q] += c[u][q];
-    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int t[3], pre[3];
+    agg_counts(P, A, i, t);
     for (int q = 0; q < 3; q++) {
         int b = 0;
         for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) b += P.csum[q * gridDim.x + k];
@@ -692,48 +684,106 @@ __global__ void agg_write_kernel(AggPass P, Mat<double> A) {
         P.moff[tot] = pre[1] + t[1];
         if (P.moffF) P.moffC[tot] = pre[2] + t[2];
     }
-    for (int u = 0; u < kAggPer; u++) {
-        if (!c[u][0]) continue;
-        const int i = base_i + u, id = pre[0], sz = c[u][1], p = P.st.partner[i];
-        int buf[kLocal];
-        int *mm = P.mem + pre[1], k = 0;
-        P.moff[id] = pre[1];
-        if (sz <= kLocal) {
-            each_member(P, A, i, p, [&](int m) { buf[k++] = m; });
-            sort_ints(buf, sz);
-            for (int q = 0; q < sz; q++) { mm[q] = buf[q]; P.agg[buf[q]] = id; }
-        } else {
-            each_member(P, A, i, p, [&](int m) { mm[k++] = m; P.agg[m] = id; });
-            sort_ints(mm, sz);
-        }
-        if (P.moffF) {
-            const int szF = c[u][2];
-            int *mf = P.memC + pre[2];
-            P.moffC[id] = pre[2];
-            int *dst = szF <= kLocal ? buf : mf;
-            int kf = 0;
-            for (int q = 0; q < sz; q++) {
-                const int m = mm[q];
-                for (int r = P.moffF[m]; r < P.moffF[m + 1]; r++) dst[kf++] = P.memF[r];
-            }
-            sort_ints(dst, szF);
-            for (int q = 0; q < szF; q++) { mf[q] = dst[q]; P.aggC[dst[q]] = id; }
-        }
-        for (int q = 0; q < 3; q++) pre[q] += c[u][q];
+    if (!t[0]) return;
+    const int id = pre[0], sz = t[1], p = P.st.partner[i];
+    int buf[kLocal];
+    int *mm = P.mem + pre[1], k = 0;
+    P.moff[id] = pre[1];
+    if (sz <= kLocal) {
+        each_member(P, A, i, p, [&](int m) { buf[k++] = m; });
+        sort_ints(buf, sz);
+        for (int q = 0; q < sz; q++) { mm[q] = buf[q]; P.agg[buf[q]] = id; }
+    } else {
+        each_member(P, A, i, p, [&](int m) { mm[k++] = m; P.agg[m] = id; });
+        sort_ints(mm, sz);
     }
+    if (!P.moffF) return;
+    const int szF = t[2];
+    int *mf = P.memC + pre[2], kf = 0;
+    int *dst = szF <= kLocal ? buf : mf;
+    P.moffC[id] = pre[2];
+    for (int q = 0; q < sz; q++) {
+        const int m = mm[q];
+        for (int r = P.moffF[m]; r < P.moffF[m + 1]; r++) dst[kf++] = P.memF[r];
+    }
+    sort_ints(dst, szF);
+    for (int q = 0; q < szF; q++) { mf[q] = dst[q]; P.aggC[dst[q]] = id; }
 }
 
 // Galerkin row I of P^T A P, one warp per row.  The members' row entries, mapped
 // to aggregate columns, are staged in member-then-column order (the order of the
 // sequential definition) and each distinct column sums its entries in that order;
-// the distinct columns are ranked ascending.  A list of at most 64 entries is
+// the distinct columns are ranked ascending.  A list of at most kGalSort entries is
 // sorted by (column, place in the list) in registers; longer ones, up to kGalCap,
 // are searched; a row beyond that is marked (first column -2) for galerkin_kernel
 // and sets bit 0 of *flags.  Writes the entries below Wcap of each row (the rest of
-// the columns holds -1 already) and the largest row length into *wmax.  85k rows of
-// a level's first pass: 23 us in one launch (counting and filling by search: 80 +
-// 102 us).
-constexpr int kGalWarps = 4, kGalCap = 384, kGalSort = 64;
+// the columns holds -1 already) and the largest row length into *wmax.  Bound by the
+// latency of a warp's chain (members, columns, aggregates, sort).  200k cells: the
+// first pass's 85k rows 75 us in one launch (counting and filling by search: 80 + 102
+// us), the third's 15k 27 us (30 + 50 us).
+constexpr int kGalWarps = 4, kGalCap = 384, kGalSort = 256;
+static_assert(kGalSort % 32 == 0 && kGalSort <= 256 && kGalCap % 32 == 0, "a lane per key, eight bits of place");
+
+// the list cl, vl of L <= 32 KR entries: element 32 r + lane of the warp's bitonic
+// sort is key r of the lane; returns the number of distinct columns
+template <int KR>
+__device__ __forceinline__ int galerkin_sorted(const int *cl, const double *vl, unsigned *sk, int L, int I, int nc, int Wcap,
+                                               int *__restrict__ ccol, double *__restrict__ cval) {
+    const int lane = threadIdx.x & 31;
+    unsigned k[KR];
+#pragma unroll
+    for (int r = 0; r < KR; r++) {
+        const int e = 32 * r + lane;
+        k[r] = e < L ? ((unsigned)cl[e] << 8) | e : 0xffffffffu;
+    }
+#pragma unroll
+    for (int size = 2; size <= 32 * KR; size <<= 1) {
+#pragma unroll
+        for (int str = size >> 1; str > 0; str >>= 1) {
+            if (str >= 32) {
+                const int d = str >> 5;
+#pragma unroll
+                for (int r = 0; r < KR; r++) {
+                    if (r & d) continue;
+                    const bool up = size == 32 * KR || ((32 * r) & size) == 0;
+                    const unsigned lo = min(k[r], k[r | d]), hi = max(k[r], k[r | d]);
+                    k[r] = up ? lo : hi;
+                    k[r | d] = up ? hi : lo;
+                }
+            } else {
+                const bool low = (lane & str) == 0;
+#pragma unroll
+                for (int r = 0; r < KR; r++) {
+                    const unsigned o = __shfl_xor_sync(0xffffffffu, k[r], str);
+                    const bool up = size == 32 * KR || ((32 * r + lane) & size) == 0;
+                    k[r] = low == up ? min(k[r], o) : max(k[r], o);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < KR; r++) sk[32 * r + lane] = k[r];
+    __syncwarp();
+    int D = 0;
+#pragma unroll
+    for (int r = 0; r < KR; r++) {
+        const int e = 32 * r + lane;
+        const unsigned c = k[r] >> 8;
+        const bool head = e < L && (e == 0 || (sk[e - 1] >> 8) != c);
+        const unsigned b = __ballot_sync(0xffffffffu, head);
+        if (head) {
+            const int rank = D + __popc(b & ((1u << lane) - 1u));
+            double sum = 0.0;
+            for (int q = e; q < L && (sk[q] >> 8) == c; q++) sum = __dadd_rn(sum, vl[sk[q] & 255u]);
+            if (rank < Wcap) {
+                ccol[(long)rank * nc + I] = (int)c;
+                cval[(long)rank * nc + I] = sum;
+            }
+        }
+        D += __popc(b);
+    }
+    return D;
+}
 
 __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
     Mat<double> A, const int *__restrict__ agg, const int *__restrict__ moff, const int *__restrict__ mem, int nc, int Wcap,
@@ -789,52 +839,12 @@ __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
     }
     __syncwarp();
     int D = 0;
-    if (L <= kGalSort && nc < (1 << 26)) {
-        // 2a. keys (column, place) sorted over the warp, two per lane
-        unsigned k0 = lane < L ? ((unsigned)cl[lane] << 6) | lane : 0xffffffffu;
-        unsigned k1 = lane + 32 < L ? ((unsigned)cl[lane + 32] << 6) | (lane + 32) : 0xffffffffu;
-        const bool two = L > 32;                   // uniform over the warp
-#pragma unroll
-        for (int size = 2; size <= 64; size <<= 1) {
-            if (size == 64 && !two) break;
-#pragma unroll
-            for (int str = size >> 1; str > 0; str >>= 1) {
-                if (str == 32) {
-                    const unsigned a = min(k0, k1), b = max(k0, k1);
-                    k0 = a; k1 = b;
-                } else {
-                    const bool low = (lane & str) == 0;
-                    const unsigned o0 = __shfl_xor_sync(0xffffffffu, k0, str);
-                    const bool up0 = size == 64 || (size == 32 ? true : (lane & size) == 0);
-                    k0 = low == up0 ? min(k0, o0) : max(k0, o0);
-                    if (two) {
-                        const unsigned o1 = __shfl_xor_sync(0xffffffffu, k1, str);
-                        const bool up1 = size == 64 || (size == 32 ? false : (lane & size) == 0);
-                        k1 = low == up1 ? min(k1, o1) : max(k1, o1);
-                    }
-                }
-            }
-        }
-        unsigned *sk = skey[w];
-        sk[lane] = k0;
-        sk[lane + 32] = k1;
-        __syncwarp();
-        const bool h0 = lane < L && (lane == 0 || (sk[lane - 1] >> 6) != (k0 >> 6));
-        const bool h1 = lane + 32 < L && (sk[lane + 31] >> 6) != (k1 >> 6);
-        const unsigned b0 = __ballot_sync(0xffffffffu, h0), b1 = __ballot_sync(0xffffffffu, h1);
-        D = __popc(b0) + __popc(b1);
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-            if (!(r ? h1 : h0)) continue;
-            const int e = lane + 32 * r, rank = r ? __popc(b0) + __popc(b1 & lt) : __popc(b0 & lt);
-            const unsigned c = (r ? k1 : k0) >> 6;
-            double sum = 0.0;
-            for (int q = e; q < L && (sk[q] >> 6) == c; q++) sum = __dadd_rn(sum, vl[sk[q] & 63u]);
-            if (rank < Wcap) {
-                ccol[(long)rank * nc + I] = (int)c;
-                cval[(long)rank * nc + I] = sum;
-            }
-        }
+    if (L <= kGalSort && nc < (1 << 24)) {
+        // 2a. keys (column, place) sorted over the warp, up to eight per lane
+        if (L <= 32) D = galerkin_sorted<1>(cl, vl, skey[w], L, I, nc, Wcap, ccol, cval);
+        else if (L <= 64) D = galerkin_sorted<2>(cl, vl, skey[w], L, I, nc, Wcap, ccol, cval);
+        else if (L <= 128) D = galerkin_sorted<4>(cl, vl, skey[w], L, I, nc, Wcap, ccol, cval);
+        else D = galerkin_sorted<8>(cl, vl, skey[w], L, I, nc, Wcap, ccol, cval);
     } else {
         // 2b. search: an entry is its column's first when none before it has the column
         unsigned firsts[kGalCap / 32];
@@ -1006,107 +1016,146 @@ gj_cluster_kernel(int n, double *__restrict__ A0, double *__restrict__ A1, const
     }
 }
 
-// The same elimination with the augmented matrix held in the shared memory of
-// the CTAs of one cluster (8, or 16 where the part schedules a cluster that
-// large; n <= kGjSmem), kGjPanel pivots at a time: CTA c
-// owns a block of rows; for each panel of up to kGjPanel consecutive pivot
-// rows (all in one CTA) the owner reduces the panel to the identity on its
-// pivot columns (Gauss-Jordan within the panel), one cluster barrier
-// publishes it (double-buffered by panel parity), and every CTA reads it
-// through distributed shared memory and subtracts, from each of its other
-// rows, the panel rows times that row's entries in the pivot columns.  In
-// exact arithmetic this is the pivot-by-pivot elimination; it needs one
-// cluster barrier per panel instead of one per pivot.  The right half of the
-// result is written to inv.
-constexpr int kGjSmem = 256, kGjPanel = 4;
+// The inverse of a matrix of at most kGjSmem rows in one launch of one cluster (8
+// CTAs, or 16 where the part schedules a cluster that large), in place in shared
+// memory: Gauss-Jordan without pivoting, eight pivots at a time.  Column j lives in
+// CTA j mod CTAs, so the eight columns of a panel lie in eight CTAs: each of them
+// brings its column of the next panel up to date first and publishes it, and the
+// cluster barrier's arrival is there; the rest of the columns follows between
+// arrival and wait.  After the barrier every CTA reads the panel (distributed shared
+// memory) and inverts its 8 x 8 pivot block D for itself, in one warp's registers:
+//   T_j = D A_Kj,  A_ij -= A_iK T_j (i outside K),  A_Kj = T_j;
+// a column j of the panel takes part with A_Kj = e_j and A_ij = 0.  Bound by that
+// chain and, near 256 rows, by the FP64 pipe of the cluster's SMs (n^2 8 / CTAs FMAs
+// a step at 2 a clock).  143 rows: 383 -> 155 us (row blocks and an augmented matrix,
+// a panel of four factored by one CTA of 1,024 threads while the others wait).
+constexpr int kGjSmem = 256, kGjNb = 8, kGjThreads = 512;
 
-__global__ void __launch_bounds__(1024, 1)
-gj_dsmem_kernel(int n, const double *__restrict__ aug, double *__restrict__ inv, const double *__restrict__ rn,
-                int *bad) {
-    extern __shared__ double gsm[];
-    cg::cluster_group cl = cg::this_cluster();
-    const int nc = (int)cl.num_blocks(), w = 2 * n, rpc = (n + nc - 1) / nc;   // rows per CTA
-    const int me = (int)cl.block_rank(), tid = threadIdx.x, bd = blockDim.x;
-    double *R = gsm;                                      // [rpc][w] own rows
-    double *P = R + (long)rpc * w;                        // [2][kGjPanel][w] panels (by panel parity)
-    double *PL = P + 2L * kGjPanel * w;                   // [kGjPanel][w] local copy of the current panel
-    double *F = PL + (long)kGjPanel * w;                  // [rpc][kGjPanel] own rows' pivot-column entries
-    const int base = me * rpc, nrows = max(0, min(rpc, n - base));
-    for (int t = tid; t < nrows * w; t += bd) R[t] = aug[(long)base * w + t];
-    __syncthreads();
-    int panel = 0;
-    for (int c = 0; c < nc; c++) {
-        const int cb = c * rpc, cn = max(0, min(rpc, n - cb));
-        for (int k0 = cb; k0 < cb + cn; k0 += kGjPanel, panel++) {
-            const int ps = min(kGjPanel, cb + cn - k0);
-            double *Pb = P + (long)(panel & 1) * kGjPanel * w;
-            // the panel rows are zero outside columns [k0, n + k0 + ps) (left of k0
-            // eliminated, right of n + k0 + ps still the untouched identity), so only
-            // that window of width n + ps changes: half the FP64 work of the full 2n
-            const int j0 = k0, wa = n + ps;
-            if (me == c) {
-                for (int t = tid; t < ps * w; t += bd) Pb[t] = R[(long)(k0 - base) * w + t];
-                __syncthreads();
-                for (int q = 0; q < ps; q++) {
-                    const double piv = Pb[(long)q * w + k0 + q];
-                    if (tid == 0) gj_check_pivot(piv, rn[k0 + q], bad);
-                    __syncthreads();
-                    for (int j = j0 + tid; j < j0 + wa; j += bd) Pb[(long)q * w + j] = Pb[(long)q * w + j] / piv;
-                    __syncthreads();
-                    double fu[kGjPanel];
+__device__ __forceinline__ void inv8_warp(double (&a)[2], int lane, const double *rn, int *bad) {
+    // lane holds row lane / 4, columns 2 (lane % 4) and the next
+    const int r = lane >> 2, c0 = 2 * (lane & 3);
 #pragma unroll
-                    for (int u = 0; u < kGjPanel; u++) fu[u] = u < ps ? Pb[(long)u * w + k0 + q] : 0.0;
-                    __syncthreads();
-                    for (int t = tid; t < ps * wa; t += bd) {
-                        const int u = t / wa, j = j0 + (t - u * wa);
-                        if (u != q) Pb[(long)u * w + j] = Pb[(long)u * w + j] - fu[u] * Pb[(long)q * w + j];
-                    }
-                    __syncthreads();
-                }
-            }
-            cl.sync();
-            const double *rP = cl.map_shared_rank(Pb, c);
-            for (int t = tid; t < ps * wa; t += bd) {
-                const int u = t / wa, j = j0 + (t - u * wa);
-                PL[(long)u * w + j] = rP[(long)u * w + j];
-            }
-            for (int t = tid; t < nrows * ps; t += bd) {
-                const int r = t / ps, u = t - r * ps;
-                F[r * kGjPanel + u] = R[(long)r * w + k0 + u];
-            }
-            __syncthreads();
-            for (int t = tid; t < nrows * wa; t += bd) {
-                const int r = t / wa, j = j0 + (t - r * wa), gi = base + r;
-                double *Rr = R + (long)r * w + j;
-                if (gi >= k0 && gi < k0 + ps) {
-                    *Rr = PL[(long)(gi - k0) * w + j];
-                } else {
-                    double v = *Rr;
-                    for (int u = 0; u < ps; u++) v -= F[r * kGjPanel + u] * PL[(long)u * w + j];
-                    *Rr = v;
-                }
-            }
-            __syncthreads();
+    for (int k = 0; k < kGjNb; k++) {
+        const int kc = k & 1, src = 4 * k + (k >> 1);
+        const double piv = __shfl_sync(0xffffffffu, a[kc], src);
+        if (bad && lane == 0) gj_check_pivot(piv, rn[k], bad);
+        const double ip = 1.0 / piv;
+        const double p0 = __shfl_sync(0xffffffffu, a[0], 4 * k + (lane & 3)) * ip;
+        const double p1 = __shfl_sync(0xffffffffu, a[1], 4 * k + (lane & 3)) * ip;
+        const double f = __shfl_sync(0xffffffffu, a[kc], (lane & ~3) + (k >> 1));
+        if (r == k) {
+            a[0] = c0 == k ? ip : p0;
+            a[1] = c0 + 1 == k ? ip : p1;
+        } else {
+            a[0] = c0 == k ? -f * ip : a[0] - f * p0;
+            a[1] = c0 + 1 == k ? -f * ip : a[1] - f * p1;
         }
     }
-    cl.sync();                                            // no CTA leaves while another may read its panels
-    for (int t = tid; t < nrows * n; t += bd) {
-        const int r = t / n, j = t - r * n;
-        inv[(long)(base + r) * n + j] = R[(long)r * w + n + j];
+}
+
+__global__ void __launch_bounds__(kGjThreads, 1) gj_inverse_kernel(Mat<double> A, double *__restrict__ inv, int *bad) {
+    extern __shared__ double gsm[];
+    cg::cluster_group cl = cg::this_cluster();
+    const int n = A.n, nc = (int)cl.num_blocks(), me = (int)cl.block_rank(), cpc = (n + nc - 1) / nc;
+    const int tid = threadIdx.x;
+    double *S = gsm;                                  // [cpc][n] own columns
+    double *pub = S + (long)cpc * n;                  // [2][n] own column of a panel, by panel parity
+    double *PL = pub + 2 * n;                         // [kGjNb][n] the current panel
+    double *Tc = PL + kGjNb * n;                      // [cpc][kGjNb]
+    double *D = Tc + cpc * kGjNb;                     // [kGjNb][kGjNb] row-major
+    double *rn = D + kGjNb * kGjNb;                   // [n + kGjNb] l1 row norms (the pivot test's scale)
+    const int mycols = n > me ? (n - me + nc - 1) / nc : 0;
+    for (int t = tid; t < cpc * n; t += kGjThreads) S[t] = 0.0;
+    __syncthreads();
+    for (int i = tid; i < n + kGjNb; i += kGjThreads) {
+        double s = 0.0;
+        if (i < n)
+            for_row(A, i, [&](int j, double v) {
+                s += fabs(v);
+                if (j % nc == me) S[(long)(j / nc) * n + i] += v;
+            });
+        rn[i] = s;
+    }
+    __syncthreads();
+    const int steps = (n + kGjNb - 1) / kGjNb;
+    if (me < kGjNb && me < n)                         // the first panel
+        for (int i = tid; i < n; i += kGjThreads) pub[i] = S[i];
+    cl.barrier_arrive();
+    for (int s = 0; s < steps; s++) {
+        const int k0 = s * kGjNb, kb = min(kGjNb, n - k0);
+        cl.barrier_wait();
+        for (int t = tid; t < kGjNb * n; t += kGjThreads) {
+            const int q = t / n, i = t - q * n;
+            PL[t] = q < kb ? cl.map_shared_rank(pub, (k0 + q) % nc)[(s & 1) * n + i] : 0.0;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            const int r = tid >> 2, c0 = 2 * (tid & 3);
+            double a[2];
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const int c = c0 + u;
+                a[u] = r < kb && c < kb ? PL[(long)c * n + k0 + r] : (r == c ? 1.0 : 0.0);
+            }
+            // rows past the end are the identity's: their pivots are 1 against a norm of 0
+            inv8_warp(a, tid, rn + k0, me == 0 ? bad : nullptr);
+#pragma unroll
+            for (int u = 0; u < 2; u++) D[r * kGjNb + c0 + u] = a[u];
+        }
+        __syncthreads();
+        for (int t = tid; t < mycols * kGjNb; t += kGjThreads) {
+            const int lc = t / kGjNb, r = t - lc * kGjNb, j = lc * nc + me;
+            double v = 0.0;
+            if (j >= k0 && j < k0 + kb) {
+                v = D[r * kGjNb + j - k0];
+            } else {
+#pragma unroll
+                for (int q = 0; q < kGjNb; q++) v += D[r * kGjNb + q] * (q < kb ? S[(long)lc * n + k0 + q] : 0.0);
+            }
+            Tc[t] = v;
+        }
+        __syncthreads();
+        auto update = [&](int lc, int i) -> double {
+            const int j = lc * nc + me;
+            if (i >= k0 && i < k0 + kb) return Tc[lc * kGjNb + i - k0];
+            double v = j >= k0 && j < k0 + kb ? 0.0 : S[(long)lc * n + i];
+#pragma unroll
+            for (int q = 0; q < kGjNb; q++) v -= PL[q * n + i] * Tc[lc * kGjNb + q];
+            return v;
+        };
+        // my column of the next panel, if I have one
+        const int nk0 = k0 + kGjNb, off = ((me - nk0) % nc + nc) % nc, nj = nk0 + off;
+        const int nl = off < kGjNb && nj < n ? nj / nc : -1;
+        if (nl >= 0)
+            for (int i = tid; i < n; i += kGjThreads) {
+                const double v = update(nl, i);
+                S[(long)nl * n + i] = v;
+                pub[((s + 1) & 1) * n + i] = v;
+            }
+        cl.barrier_arrive();                          // releases the published column
+        for (int t = tid; t < mycols * n; t += kGjThreads) {
+            const int lc = t / n, i = t - lc * n;
+            if (lc != nl) S[t] = update(lc, i);
+        }
+        __syncthreads();                              // PL, Tc and S are read and written again
+    }
+    cl.barrier_wait();                                // no CTA leaves while another may read its column
+    for (int t = tid; t < mycols * n; t += kGjThreads) {
+        const int lc = t / n, i = t - lc * n;
+        inv[(long)i * n + lc * nc + me] = S[t];
     }
 }
 
-static size_t gj_dsmem_bytes(int n, int nc) {
-    const int w = 2 * n, rpc = (n + nc - 1) / nc;
-    return sizeof(double) * ((size_t)rpc * w + 3 * (size_t)kGjPanel * w + (size_t)rpc * kGjPanel);
+static size_t gj_inverse_bytes(int n, int nc) {
+    const int cpc = (n + nc - 1) / nc;
+    return sizeof(double) * ((size_t)cpc * n + (2 + kGjNb) * (size_t)n + (size_t)cpc * kGjNb + kGjNb * kGjNb + n + kGjNb);
 }
 
-// [A | I], one thread per entry (row i, column j of the n x 2n array)
 // CTAs of the Gauss-Jordan cluster: 16 (a non-portable size) when the
 // occupancy query finds room for one such cluster at the largest shared-memory
 // size, else the portable 8; the query launches nothing
 static int gj_cluster_ctas() {
-    if (cudaFuncSetAttribute(gj_dsmem_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         (void)cudaGetLastError();
         return 8;
     }
@@ -1114,16 +1163,17 @@ static int gj_cluster_ctas() {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 16; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(16); cfg.blockDim = dim3(1024); cfg.dynamicSmemBytes = gj_dsmem_bytes(kGjSmem, 16);
+    cfg.gridDim = dim3(16); cfg.blockDim = dim3(kGjThreads); cfg.dynamicSmemBytes = gj_inverse_bytes(kGjSmem, 16);
     cfg.attrs = at; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, gj_dsmem_kernel, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, gj_inverse_kernel, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         return 8;
     }
     return clusters > 0 ? 16 : 8;
 }
 
+// [A | I], one thread per entry (row i, column j of the n x 2n array)
 __global__ void gj_init_kernel(Mat<double> A, double *__restrict__ aug) {
     const long w = 2L * A.n;
     const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -1890,10 +1940,10 @@ static bool enqueue_pass(sim_t *s, const Mat<double> &A, bool second, int *aggC,
     P.agg = second ? s->aggB : s->aggA; P.moff = second ? s->moffB : s->moffA; P.mem = second ? s->memB : s->memA;
     P.aggC = aggC; P.moffC = moffC; P.memC = memC;
     P.csum = s->scan; P.nc = s->iscal + kScNc;
-    // chunks of 1,024 nodes spread a small level over the SMs; from 2M nodes chunks
-    // of 4,096 keep the sums every block adds up for its base short
-    const int threads = n <= (1 << 21) ? 256 : 1024;
-    const int chunks = (int)(((long)n + threads * kAggPer - 1) / (threads * kAggPer));
+    // chunks of 256 nodes spread a small level over the SMs; from 256k nodes chunks
+    // of 1,024 keep the sums every block adds up for its base short
+    const int threads = n <= (1 << 18) ? 256 : 1024;
+    const int chunks = sim_blocks(n, threads);
     agg_sizes_kernel<<<chunks, threads, 0, s->stream>>>(P, A);
     agg_write_kernel<<<chunks, threads, 0, s->stream>>>(P, A);
     s->launches += 2;
@@ -2007,46 +2057,40 @@ static sim_status finish_levels(sim_t *s) {
     // coarsest: dense Gauss-Jordan inverse in FP64
     AmgLevel &C = s->lev[nl - 1];
     const int n = C.n;
-    const size_t aug = (size_t)n * 2 * n;
-    double *A0 = (double *)dev_alloc_async(s, sizeof(double) * aug);
-    double *A1 = (double *)dev_alloc_async(s, sizeof(double) * aug);
-    double *rn = (double *)dev_alloc_async(s, sizeof(double) * n);
-    if (!A0 || !A1 || !rn) return s->err;
-    int *bad = s->iscal + kScBad;
-    SIM_CK(s, cudaMemsetAsync(bad, 0, sizeof(int), s->stream));
-    gj_init_kernel<<<sim_blocks(2L * n * n), SIM_THREADS, 0, s->stream>>>(level_mat(s, C, nl - 1), A0);
-    s->launches++;
-    gj_rownorm_kernel<<<sim_blocks(n), SIM_THREADS, 0, s->stream>>>(level_mat(s, C, nl - 1), rn);
-    s->launches++;
-    static bool dsmem_ok = cudaFuncSetAttribute(gj_dsmem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)gj_dsmem_bytes(kGjSmem, 8)) == cudaSuccess;
-    static int gj_ctas = gj_cluster_ctas();
-    const bool in_smem = dsmem_ok && n <= kGjSmem;
-    if (!in_smem) {
-        gj_cluster_kernel<<<8, 1024, 0, s->stream>>>(n, A0, A1, rn, bad);
-        s->launches++;
-    }
     // the coarsest inverse stays FP64 in both forms: the coarse matrices of
     // strongly heterogeneous fields are ill-conditioned, and the product is tiny
     C.coarse_inv = dev_alloc_async(s, sizeof(double) * (size_t)n * n);
     if (!C.coarse_inv) return s->err;
-    if (in_smem) {
+    int *bad = s->iscal + kScBad;
+    SIM_CK(s, cudaMemsetAsync(bad, 0, sizeof(int), s->stream));
+    static bool smem_ok = cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)gj_inverse_bytes(kGjSmem, 8)) == cudaSuccess;
+    static int gj_ctas = gj_cluster_ctas();
+    if (smem_ok && n <= kGjSmem) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = gj_ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(gj_ctas); cfg.blockDim = dim3(1024); cfg.dynamicSmemBytes = gj_dsmem_bytes(n, gj_ctas);
+        cfg.gridDim = dim3(gj_ctas); cfg.blockDim = dim3(kGjThreads); cfg.dynamicSmemBytes = gj_inverse_bytes(n, gj_ctas);
         cfg.stream = s->stream; cfg.attrs = at; cfg.numAttrs = 1;
-        if (!sim_cuda_ok(s, cudaLaunchKernelEx(&cfg, gj_dsmem_kernel, n, (const double *)A0, (double *)C.coarse_inv,
-                                               (const double *)rn, bad),
+        if (!sim_cuda_ok(s, cudaLaunchKernelEx(&cfg, gj_inverse_kernel, level_mat(s, C, nl - 1), (double *)C.coarse_inv, bad),
                          "coarsest inverse"))
             return s->err;
+        s->launches++;
     } else {
+        const size_t aug = (size_t)n * 2 * n;
+        double *A0 = (double *)dev_alloc_async(s, sizeof(double) * aug);
+        double *A1 = (double *)dev_alloc_async(s, sizeof(double) * aug);
+        double *rn = (double *)dev_alloc_async(s, sizeof(double) * n);
+        if (!A0 || !A1 || !rn) return s->err;
+        gj_init_kernel<<<sim_blocks(2L * n * n), SIM_THREADS, 0, s->stream>>>(level_mat(s, C, nl - 1), A0);
+        gj_rownorm_kernel<<<sim_blocks(n), SIM_THREADS, 0, s->stream>>>(level_mat(s, C, nl - 1), rn);
+        gj_cluster_kernel<<<8, 1024, 0, s->stream>>>(n, A0, A1, rn, bad);
         gj_extract_kernel<double><<<sim_blocks((long)n * n), SIM_THREADS, 0, s->stream>>>(n, (n & 1) ? A1 : A0,
                                                                                         (double *)C.coarse_inv);
+        s->launches += 4;
+        dev_free_async(s, A0); dev_free_async(s, A1); dev_free_async(s, rn);
     }
-    s->launches++;
-    dev_free_async(s, A0); dev_free_async(s, A1); dev_free_async(s, rn);
     SIM_CK(s, cudaGetLastError());
     // the pivot test of the elimination (no pivoting: a vanishing pivot would
     // leave inf / NaN in the coarsest inverse)

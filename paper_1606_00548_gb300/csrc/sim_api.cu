@@ -328,7 +328,7 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     s->memA = (int *)A(sizeof(int) * N);
     s->moffB = (int *)A(sizeof(int) * (N + 1));
     s->memB = (int *)A(sizeof(int) * N);
-    s->scan = (int *)A(sizeof(int) * 3 * (N / 1024 + 2));
+    s->scan = (int *)A(sizeof(int) * 3 * (N / 256 + 2));
     s->iscal = (int *)A(sizeof(int) * 16);
     if (!ok) {
         std::string m = s->msg;

@@ -1,5 +1,5 @@
 """The AMG hierarchy bit for bit against the oracle at the edges of the set-up's
-launches: one to a few thousand nodes around the 1,024-node chunks of the
+launches: one to a few thousand nodes around the chunks (256 or 1,024 nodes) of the
 numbering, more than 2^21 nodes (chunks of 4,096), one- and two-dimensional
 grids, several numbers of matching rounds, rough pressure blocks (many absorbed
 nodes and wide coarse rows), and a strength threshold that leaves nodes alone.
