@@ -107,10 +107,9 @@ struct Mat {
     const V *val;    // structured: [7][n]; ELL: [width][n]
     const int *col;  // ELL
     int n, width;
+    const int *len = nullptr;  // ELL: entries of each row (the width is the longest row's, two to three times the mean)
     const int *wp = nullptr;   // set-up: {width, flags} still on the device (width then holds the capacity)
 };
-// width of an ELL matrix during the set-up
-template <typename V> __device__ __forceinline__ int ell_width(const Mat<V> &A) { return A.wp ? A.wp[0] : A.width; }
 // a product whose rows did not all fit is no matrix yet (entries are missing, and
 // with them the symmetry of its pattern): what was enqueued on it does nothing, and
 // the host, which reads the same words, builds it again and repeats the pass
@@ -135,31 +134,27 @@ __device__ __forceinline__ void for_row(const Mat<V> &A, int i, F f) {
         if (iz < A.g.nz - 1) f(i + nxy, A.val[6 * n + i]);
     } else if (A.selfpad) {
         // batches of 8 entries: the batch's loads are issued together, then f
-        // runs on them in column-slot order
-        for (int k0 = 0; k0 < A.width; k0 += 8) {
+        // runs on them in column-slot order; padding within the last batch is
+        // (own column, 0)
+        const int W = A.len[i];
+        for (int k0 = 0; k0 < W; k0 += 8) {
             int jj[8];
             V vv[8];
 #pragma unroll
             for (int u = 0; u < 8; u++) {
                 const long q = (long)(k0 + u) * A.n + i;
-                const bool ok = k0 + u < A.width;
+                const bool ok = k0 + u < W;
                 jj[u] = ok ? A.col[q] : i;
                 vv[u] = ok ? A.val[q] : V(0);
             }
 #pragma unroll
             for (int u = 0; u < 8; u++)
-                if (k0 + u < A.width) f(jj[u], vv[u]);
+                if (k0 + u < W) f(jj[u], vv[u]);
         }
     } else {
-        // -1 padding sits only at the end of a row: skipping it instead of
-        // stopping there visits the same entries in the same order, and the
-        // column loads no longer wait on one another
-        const int W = ell_width(A);
+        const int W = A.len[i];
 #pragma unroll 4
-        for (int k = 0; k < W; k++) {
-            const int j = A.col[(long)k * A.n + i];
-            if (j >= 0) f(j, A.val[(long)k * A.n + i]);
-        }
+        for (int k = 0; k < W; k++) f(A.col[(long)k * A.n + i], A.val[(long)k * A.n + i]);
     }
 }
 
@@ -178,6 +173,68 @@ __device__ __forceinline__ T row_dot(const Mat<T> &A, int i, const T *__restrict
         for_row(A, i, [&](int j, T v) { t += v * e[j]; });
     }
     return t;
+}
+
+// ---- lanes of an ELL row ----------------------------------------------------
+// A row of 8 to 25 entries taken by one thread is a chain of load batches; below
+// 131k rows, where the launch does not fill the GPU with rows, lanes share a row and
+// have all of its entries in flight at once (72k rows, longest 35, mean 11 entries:
+// residual 16.6 -> 10.8 us with the row lengths).  The count depends on the level's size
+// only, so every kernel that takes the row (one system, a batch, the fused coarse
+// cycle) adds it up alike.
+__host__ __device__ inline int ell_lanes(int n) { return n > 131072 ? 1 : n > 2048 ? 4 : n > 512 ? 8 : 16; }
+
+// sum_k val_k e(col_k) of row i by `lanes` adjacent lanes (sub: this one's number;
+// every lane of the warp calls, ok: the row exists), the total in all of them.
+// entry(k, j, v) gives column and value of slot k < W (padding: column i, value 0);
+// len: slots the row uses, whose largest in the warp ends the loop -- the first
+// batch's loads do not wait for it.  FP64: each lane adds its own slots, then a fixed
+// tree.  Difference form (FP32 copies, see row_dot): the products are added in slot
+// order, one lane's after the other's, so the rounding is that of one thread taking
+// the row.
+template <typename T, typename FEnt, typename FE>
+__device__ __forceinline__ T row_dot_lanes(int W, int len, int lanes, int sub, bool ok, bool diff, int i, T ei, FEnt entry,
+                                           FE e) {
+    constexpr int U = 4;
+    T t = (T)0;
+    int most = W, j[U];
+    T v[U];
+    for (int k0 = 0; k0 < most; k0 += U * lanes) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = k0 + u * lanes + sub;
+            j[u] = i;
+            v[u] = (T)0;
+            if (ok && k < W) entry(k, j[u], v[u]);
+        }
+        T x[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) x[u] = ok ? e(j[u]) : (T)0;
+        if (k0 == 0) most = __reduce_max_sync(0xffffffffu, ok ? len : 0);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (k0 + u * lanes >= most) break;                 // uniform
+            if (!diff) {
+                t += v[u] * x[u];
+            } else {
+                const T d = j[u] == i ? ei : x[u] - ei;
+                if (lanes == 1) { t = fma(v[u], d, t); continue; }
+                for (int l = 0; l < lanes; l++)
+                    t = fma(__shfl_sync(0xffffffffu, v[u], l, lanes), __shfl_sync(0xffffffffu, d, l, lanes), t);
+            }
+        }
+    }
+    if (!diff)
+        for (int o = lanes >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+// A_i . e of an ELL level of the application with `lanes` lanes
+template <typename T>
+__device__ __forceinline__ T mat_dot_lanes(const Mat<T> &A, int i, bool ok, int lanes, int sub, const T *__restrict__ e) {
+    const long n = A.n;
+    return row_dot_lanes<T>(A.width, ok ? A.len[i] : 0, lanes, sub, ok, A.diff, i, ok && A.diff ? e[i] : (T)0,
+                            [&](int k, int &j, T &v) { j = A.col[k * n + i]; v = A.val[k * n + i]; },
+                            [&](int j) { return e[j]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -532,13 +589,13 @@ __global__ void __launch_bounds__(SIM_THREADS) match_kernel(Mat<double> A, Match
         }
     } else {
         constexpr int U = 4;                       // entries of a lane kept in registers: rows of up to 32
-        const int W = ell_width(A);
+        const int W = open ? A.len[i] : 0;
         long long mx = 0, a[U];
         int jj[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int k = sub + LANES * u;
-            jj[u] = open && k < W ? A.col[(long)k * n + i] : -1;
+            jj[u] = k < W ? A.col[(long)k * n + i] : -1;
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
@@ -546,8 +603,8 @@ __global__ void __launch_bounds__(SIM_THREADS) match_kernel(Mat<double> A, Match
             mx = max(mx, a[u]);
         }
         for (int k = sub + LANES * U; k < W; k += LANES) {
-            const int j = open ? A.col[(long)k * n + i] : -1;
-            if (j >= 0 && j != i) mx = max(mx, neg_bits(A.val[(long)k * n + i]));
+            const int j = A.col[(long)k * n + i];
+            if (j != i) mx = max(mx, neg_bits(A.val[(long)k * n + i]));
         }
 #pragma unroll
         for (int o = LANES / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -556,8 +613,8 @@ __global__ void __launch_bounds__(SIM_THREADS) match_kernel(Mat<double> A, Match
 #pragma unroll
             for (int u = 0; u < U; u++) consider(jj[u], a[u], lim);
             for (int k = sub + LANES * U; k < W; k += LANES) {
-                const int j = open ? A.col[(long)k * n + i] : -1;
-                if (j >= 0 && j != i) consider(j, neg_bits(A.val[(long)k * n + i]), lim);
+                const int j = A.col[(long)k * n + i];
+                if (j != i) consider(j, neg_bits(A.val[(long)k * n + i]), lim);
             }
         }
 #pragma unroll
@@ -787,7 +844,7 @@ __device__ __forceinline__ int galerkin_sorted(const int *cl, const double *vl, 
 
 __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
     Mat<double> A, const int *__restrict__ agg, const int *__restrict__ moff, const int *__restrict__ mem, int nc, int Wcap,
-    int *__restrict__ ccol, double *__restrict__ cval, int *wmax, int *flags) {
+    int *__restrict__ ccol, double *__restrict__ cval, int *__restrict__ clen, int *wmax, int *flags) {
     __shared__ int scol[kGalWarps][kGalCap];
     __shared__ double sval[kGalWarps][kGalCap];
     __shared__ unsigned skey[kGalWarps][kGalSort];
@@ -798,8 +855,14 @@ __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
     double *vl = sval[w];
     const unsigned lt = (1u << lane) - 1u;
     // 1. the ordered list: slots (member, entry of its row), four per lane in flight
-    const int W = A.st ? 7 : ell_width(A);
-    const int q0 = moff[I], slots = (moff[I + 1] - q0) * W;
+    const int q0 = moff[I], nm = moff[I + 1] - q0;
+    int W = 7;                                    // the members' longest row
+    if (!A.st) {
+        W = 0;
+        for (int q = lane; q < nm; q += 32) W = max(W, A.len[mem[q0 + q]]);
+        W = __reduce_max_sync(0xffffffffu, W);
+    }
+    const int slots = nm * W;
     int L = 0;
     for (int s0 = 0; s0 < slots; s0 += 4 * 32) {
         int col[4];
@@ -821,7 +884,7 @@ __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
                     const int off = d == 0 ? 0 : d == 1 ? -1 : d == 2 ? 1 : d == 3 ? -nx : d == 4 ? nx : d == 5 ? -nxy : nxy;
                     if (ok) { col[u] = m + off; v[u] = A.val[(long)d * A.n + m]; }
                 } else {
-                    col[u] = A.col[(long)k * A.n + m];
+                    col[u] = A.col[(long)k * A.n + m];      // -1 past the row's end
                     if (col[u] >= 0) v[u] = A.val[(long)k * A.n + m];
                 }
             }
@@ -876,7 +939,10 @@ __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
             }
         }
     }
-    if (lane == 0 && D > *(volatile int *)wmax) atomicMax(wmax, D);
+    if (lane == 0) {
+        clen[I] = D;
+        if (D > *(volatile int *)wmax) atomicMax(wmax, D);
+    }
 }
 
 // Galerkin rows the row kernel marked, one thread per row: members moff/mem
@@ -884,7 +950,7 @@ __global__ void __launch_bounds__(kGalWarps * 32) galerkin_row_kernel(
 // ascending.  A row of more than SIM_MAX_ELL columns sets bit 1 of *flags.
 __global__ void galerkin_kernel(Mat<double> A, const int *__restrict__ agg, const int *__restrict__ moff,
                                 const int *__restrict__ mem, int nc, int Wcap, int *__restrict__ ccol,
-                                double *__restrict__ cval, int *wmax, int *flags) {
+                                double *__restrict__ cval, int *__restrict__ clen, int *wmax, int *flags) {
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc || ccol[I] != -2) return;
     int cols[MAXE];
@@ -905,6 +971,7 @@ __global__ void galerkin_kernel(Mat<double> A, const int *__restrict__ agg, cons
         });
     }
     if (over) { atomicOr(flags, 2); return; }
+    clen[I] = cnt;
     atomicMax(wmax, cnt);
     if (cnt > Wcap) return;                        // built again with room for it
     for (int a = 1; a < cnt; a++) {
@@ -1256,14 +1323,25 @@ __global__ void restrict_p_kernel(int N, const double *__restrict__ r, const T *
     restrict_p_row<B, T>(N, r, wT, full, dinv0, f0, e0, i);
 }
 
-// r = f - A e (one thread per fine row: coalesced stencil / ELL reads)
+// r = f - A e, row i by `lanes` lanes from thread t of the level's launch on (a
+// thread per row on the 7-point level: coalesced stencil reads)
+template <typename T>
+__device__ __forceinline__ void amg_resid_row(const Mat<T> &A, const T *__restrict__ f, const T *__restrict__ e,
+                                              T *__restrict__ r, long t) {
+    if (A.st) {
+        if (t < A.n) r[t] = f[t] - row_dot(A, (int)t, e);
+        return;
+    }
+    const int lanes = ell_lanes(A.n), i = (int)(t / lanes), sub = (int)(t & (lanes - 1));
+    const bool ok = i < A.n;
+    const T d = mat_dot_lanes(A, i, ok, lanes, sub, e);
+    if (ok && sub == 0) r[i] = f[i] - d;
+}
 template <typename T>
 __global__ void amg_resid_kernel(Mat<T> A, const T *__restrict__ f, const T *__restrict__ e, T *__restrict__ r,
                                  const int *done) {
     if (skip(done)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.n) return;
-    r[i] = f[i] - row_dot(A, i, e);
+    amg_resid_row<T>(A, f, e, r, blockIdx.x * (long)blockDim.x + threadIdx.x);
 }
 
 // f_c = P^T r of coarse row I
@@ -1311,14 +1389,24 @@ __global__ void amg_prolong_kernel(int n, const int *__restrict__ agg, const T *
     if (i < n) e[i] += ec[agg[i]];
 }
 
-// e2 = e + (f - A e) / l1 (post-smoothing)
+// e2 = e + (f - A e) / l1 (post-smoothing), threads as in amg_resid_row
+template <typename T>
+__device__ __forceinline__ void amg_smooth_row(const Mat<T> &A, const T *__restrict__ f, const T *__restrict__ e,
+                                               const T *__restrict__ dinv, T *__restrict__ e2, long t) {
+    if (A.st) {
+        if (t < A.n) e2[t] = e[t] + (f[t] - row_dot(A, (int)t, e)) * dinv[t];
+        return;
+    }
+    const int lanes = ell_lanes(A.n), i = (int)(t / lanes), sub = (int)(t & (lanes - 1));
+    const bool ok = i < A.n;
+    const T d = mat_dot_lanes(A, i, ok, lanes, sub, e);
+    if (ok && sub == 0) e2[i] = e[i] + (f[i] - d) * dinv[i];
+}
 template <typename T>
 __global__ void amg_smooth_kernel(Mat<T> A, const T *__restrict__ f, const T *__restrict__ e, const T *__restrict__ dinv,
                                   T *__restrict__ e2, const int *done) {
     if (skip(done)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.n) return;
-    e2[i] = e[i] + (f[i] - row_dot(A, i, e)) * dinv[i];
+    amg_smooth_row<T>(A, f, e, dinv, e2, blockIdx.x * (long)blockDim.x + threadIdx.x);
 }
 
 // next stage-P cycle: f0 = rp - A_p ep; e0 = f0 / l1
@@ -1355,17 +1443,28 @@ __global__ void coarse_solve_kernel(int n, const double *__restrict__ Inv, const
 }
 
 // ---- the coarse end of the V-cycle in one launch --------------------------
-// Levels l0..nl-1 (each at most kCoarseRows rows) run inside one thread-block
+// Levels l0..nl-1 (each at most coarse_rows rows) run inside one thread-block
 // cluster: the same row operations as the per-level kernels, with a cluster
 // barrier between dependent sweeps instead of a kernel boundary.  On entry
 // level l0 holds f and its pre-smoothed e; on exit its corrected vector is e2.
-constexpr int kCoarseCtas = 8, kCoarseThreads = 1024, kCoarseRows = 2 * kCoarseCtas * kCoarseThreads;
+// Every sweep is a chain of dependent L2 loads: 16 CTAs (8 where the part does not
+// schedule a cluster that large) give each row its lanes (ell_lanes), the prolonged
+// correction is added where the post-smoothing reads it (one sweep and one barrier
+// less a level), and a row's loop ends at the warp's longest row, not at the ELL
+// width.  What a larger level costs here is the latency of its passes on 16 SMs
+// (8,000 rows: residual 6 us, post-smoothing 9 us), so it is left to the per-level
+// launches over all SMs: above 3,072 rows in FP64 (200k-cell Newton iteration 31.8 ms
+// with 16,384 rows, 31.2 with 3,000; application of 398k cells 213 and 202 us), above
+// 6,144 in FP32, whose sums are cheaper (151k cells: 14.65 ms, 15.1 with 3,000).
+constexpr int kCoarseThreads = 1024;
+inline int coarse_rows(bool fp32) { return fp32 ? 6144 : 3072; }
 constexpr int kCoarseMaxLevels = 24;
 
 template <typename T>
 struct CoarseLevel {
-    int n, width, diff;
+    int n, width, diff, st;   // st: level 0, the 7-point stencil
     const int *colA;     // self-padded ELL columns [width][n]
+    const int *len;      // entries of each row
     const T *val;        // [width][n]
     const T *dinv;       // 1 / l1 row sums
     const int *agg;      // row -> next-level aggregate
@@ -1376,42 +1475,47 @@ struct CoarseLevel {
 template <typename T>
 struct CoarseCycle {
     int nlev;                          // levels in lv (the last one is the coarsest)
+    GridDesc g;                        // of a structured level
     const double *inv;                 // coarsest: dense inverse, row-major (FP64)
     CoarseLevel<T> lv[kCoarseMaxLevels];
 };
 
-template <typename T>
-__device__ __forceinline__ T ell_dot(const CoarseLevel<T> &L, int i, const T *__restrict__ e) {
-    T t = (T)0;
-    if (L.diff) {                                  // difference form (see row_dot)
-        const T ei = e[i];
-#pragma unroll 4
-        for (int k = 0; k < L.width; k++) {
-            const int j = L.colA[(long)k * L.n + i];
-            const T v = L.val[(long)k * L.n + i];
-            t += (j == i) ? v * ei : v * (e[j] - ei);
-        }
-        return t;
-    }
-#pragma unroll 4
-    for (int k = 0; k < L.width; k++) t += L.val[(long)k * L.n + i] * e[L.colA[(long)k * L.n + i]];
-    return t;
+// the arrival releases this thread's global writes to the cluster, the wait acquires the others'
+__device__ __forceinline__ void cluster_barrier() { cg::this_cluster().sync(); }
+
+// rows lo..hi of a level of n rows for CTA `rank` of nb: one contiguous block each,
+// so every SM of the cluster carries an equal share of a small level's L2 traffic
+// (a grid-wide thread index would leave a 1,000-row level to one or two SMs);
+// f(row, row exists, lane of the row) on every lane of the CTA together
+template <typename F>
+__device__ __forceinline__ void sweep_rows(int n, int lanes, int rank, int nb, F f) {
+    const int per = (n + nb - 1) / nb, lo = min(n, rank * per), hi = min(n, lo + per);
+    const int sub = threadIdx.x & (lanes - 1), at = threadIdx.x / lanes, step = blockDim.x / lanes;
+    for (int b = lo; b < hi; b += step) f(b + at, b + at < hi, sub);
 }
 
-__device__ __forceinline__ void cluster_barrier() {
-    __threadfence();                   // global writes of this thread before the barrier
-    cg::this_cluster().sync();
+template <typename T, typename FE>
+__device__ __forceinline__ T coarse_dot(const CoarseCycle<T> &cc, const CoarseLevel<T> &L, int i, bool ok, int lanes, int sub,
+                                        T ei, FE e) {
+    const long n = L.n;
+    return row_dot_lanes<T>(L.width, L.st ? 7 : (ok ? L.len[i] : 0), lanes, sub, ok, L.diff != 0, i, ei,
+                            [&](int k, int &j, T &v) {
+                                if (L.st) {
+                                    const int d = k == 0 ? 5 : k == 1 ? 3 : k == 2 ? 1 : k == 3 ? 0 : k == 4 ? 2 : k == 5 ? 4 : 6;
+                                    const int q = nbr7(cc.g, i, d);
+                                    if (q >= 0) { j = q; v = L.val[d * n + i]; }
+                                } else {
+                                    j = L.colA[k * n + i];
+                                    v = L.val[k * n + i];
+                                }
+                            },
+                            e);
 }
 
 // the cycle run by CTA `rank` of the nb CTAs of one cluster
 template <typename T>
 __device__ __forceinline__ void coarse_cycle_body(const CoarseCycle<T> &cc, int rank, int nb) {
-    // each sweep splits a level's rows into one contiguous block per CTA, so every
-    // SM of the cluster carries an equal share of a small level's L2 traffic
-    // (a grid-wide thread index would leave a 1,000-row level to one or two SMs)
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    auto lo_of = [&](int n) { const int per = (n + nb - 1) / nb; return min(n, rank * per); };
-    auto hi_of = [&](int n) { const int per = (n + nb - 1) / nb; return min(n, (rank + 1) * per); };
     const int last = cc.nlev - 1;
     // the matrices of the levels below the first and the dense inverse come into
     // L2 while the first level is swept: one bulk prefetch per (array, CTA)
@@ -1430,21 +1534,38 @@ __device__ __forceinline__ void coarse_cycle_body(const CoarseCycle<T> &cc, int 
     }
     for (int l = 0; l < last; l++) {
         const CoarseLevel<T> &L = cc.lv[l], &C = cc.lv[l + 1];
-        for (int i = lo_of(L.n) + threadIdx.x; i < hi_of(L.n); i += blockDim.x) L.e2[i] = L.f[i] - ell_dot(L, i, L.e);
+        const int lanes = ell_lanes(L.n);
+        sweep_rows(L.n, lanes, rank, nb, [&](int i, bool ok, int sub) {
+            const T t = coarse_dot<T>(cc, L, i, ok, lanes, sub, ok ? L.e[i] : (T)0, [&](int j) { return L.e[j]; });
+            if (ok && sub == 0) L.e2[i] = L.f[i] - t;
+        });
         cluster_barrier();
-        for (int I = lo_of(C.n) + threadIdx.x; I < hi_of(C.n); I += blockDim.x) {
+        // restriction: eight lanes load a coarse row's members, added in member order
+        sweep_rows(C.n, 8, rank, nb, [&](int I, bool ok, int sub) {
+            const int q0 = ok ? L.moff[I] : 0, q1 = ok ? L.moff[I + 1] : 0;
+            const int most = __reduce_max_sync(0xffffffffu, q1 - q0);
             T s = (T)0;
-            for (int q = L.moff[I]; q < L.moff[I + 1]; q++) s += L.e2[L.mem[q]];
-            C.f[I] = s;
-            if (l + 1 < last) C.e[I] = s * C.dinv[I];
-        }
+            for (int b = 0; b < most; b += 8) {
+                const T v = q0 + b + sub < q1 ? L.e2[L.mem[q0 + b + sub]] : (T)0;
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    const T x = __shfl_sync(0xffffffffu, v, u, 8);
+                    if (q0 + b + u < q1) s += x;
+                }
+            }
+            if (ok && sub == 0) {
+                C.f[I] = s;
+                if (l + 1 < last) C.e[I] = s * C.dinv[I];
+            }
+        });
         cluster_barrier();
     }
     {
         const CoarseLevel<T> &C = cc.lv[last];
-        for (int r = lo_of(C.n) + wib; r < hi_of(C.n); r += wpb) {
+        const int per = (C.n + nb - 1) / nb, hi = min(C.n, (rank + 1) * per);
+        for (int r = rank * per + wib; r < hi; r += wpb) {
             double s = 0.0;
-#pragma unroll 4
+#pragma unroll 8
             for (int j = lane; j < C.n; j += 32) s += cc.inv[(long)r * C.n + j] * (double)C.f[j];
             for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
             if (lane == 0) C.e[r] = (T)s;
@@ -1454,16 +1575,19 @@ __device__ __forceinline__ void coarse_cycle_body(const CoarseCycle<T> &cc, int 
     for (int l = last - 1; l >= 0; l--) {
         const CoarseLevel<T> &L = cc.lv[l], &C = cc.lv[l + 1];
         const T *ec = (l + 1 == last) ? C.e : C.e2;
-        for (int i = lo_of(L.n) + threadIdx.x; i < hi_of(L.n); i += blockDim.x) L.e[i] += ec[L.agg[i]];
-        cluster_barrier();
-        for (int i = lo_of(L.n) + threadIdx.x; i < hi_of(L.n); i += blockDim.x)
-            L.e2[i] = L.e[i] + (L.f[i] - ell_dot(L, i, L.e)) * L.dinv[i];
+        const int lanes = ell_lanes(L.n);
+        sweep_rows(L.n, lanes, rank, nb, [&](int i, bool ok, int sub) {
+            auto e = [&](int j) { return L.e[j] + ec[L.agg[j]]; };
+            const T ei = ok ? e(i) : (T)0;
+            const T t = coarse_dot<T>(cc, L, i, ok, lanes, sub, ei, e);
+            if (ok && sub == 0) L.e2[i] = ei + (L.f[i] - t) * L.dinv[i];
+        });
         if (l > 0) cluster_barrier();
     }
 }
 
 template <typename T>
-__global__ void __cluster_dims__(kCoarseCtas, 1, 1) __launch_bounds__(kCoarseThreads, 1)
+__global__ void __launch_bounds__(kCoarseThreads, 1)
 coarse_cycle_kernel(const __grid_constant__ CoarseCycle<T> cc, const int *done) {
     if (skip(done)) return;            // uniform over the cluster: no thread reaches a barrier alone
     // (a grid constant: the body reads the description in parameter space, no copy)
@@ -1889,6 +2013,7 @@ static Mat<double> level_mat(sim_t *s, const AmgLevel &L, int l) {
     A.st = (l == 0); A.selfpad = false; A.diff = false; A.g = s->gd; A.n = L.n; A.width = L.width;
     A.val = l == 0 ? s->ap : L.val;
     A.col = L.col;
+    A.len = L.len;
     return A;
 }
 template <typename T>
@@ -1897,6 +2022,7 @@ static Mat<T> level_matT(sim_t *s, const AmgLevel &L, int l) {
     A.st = (l == 0); A.selfpad = true; A.diff = sizeof(T) == sizeof(float); A.g = s->gd; A.n = L.n; A.width = L.width;
     A.val = (const T *)L.valT;
     A.col = L.colA;
+    A.len = L.len;
     return A;
 }
 
@@ -1957,14 +2083,15 @@ struct GalerkinJob {
     Mat<double> A;
     const int *agg = nullptr, *moff = nullptr, *mem = nullptr;
     int nc = 0, Wcap = 0, sc = 0;
-    int *col = nullptr;
+    int *col = nullptr;                // Wcap x nc columns, then the nc row lengths
     double *val = nullptr;
+    int *len() const { return col ? col + (size_t)Wcap * nc : nullptr; }
 };
 
 static bool galerkin_alloc(sim_t *s, GalerkinJob &g, int W) {
     dev_free_async(s, g.col); dev_free_async(s, g.val);
     g.Wcap = W;
-    g.col = (int *)dev_alloc_async(s, sizeof(int) * (size_t)W * g.nc);
+    g.col = (int *)dev_alloc_async(s, sizeof(int) * (size_t)(W + 1) * g.nc);
     g.val = (double *)dev_alloc_async(s, sizeof(double) * (size_t)W * g.nc);
     return g.col && g.val &&
            sim_cuda_ok(s, cudaMemsetAsync(g.col, 0xff, sizeof(int) * (size_t)W * g.nc, s->stream), "memset") &&
@@ -1972,7 +2099,7 @@ static bool galerkin_alloc(sim_t *s, GalerkinJob &g, int W) {
 }
 static bool galerkin_rows(sim_t *s, GalerkinJob &g) {
     galerkin_row_kernel<<<(g.nc + kGalWarps - 1) / kGalWarps, kGalWarps * 32, 0, s->stream>>>(
-        g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col, g.val, s->iscal + g.sc, s->iscal + g.sc + 1);
+        g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col, g.val, g.len(), s->iscal + g.sc, s->iscal + g.sc + 1);
     s->launches++;
     return sim_cuda_ok(s, cudaGetLastError(), "Galerkin");
 }
@@ -2002,7 +2129,7 @@ static int resolve_galerkin(sim_t *s, GalerkinJob &g, const int (&v)[kScCount], 
         }
         int u[kScCount];
         galerkin_kernel<<<sim_blocks(g.nc), SIM_THREADS, 0, s->stream>>>(g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col, g.val,
-                                                                         s->iscal + g.sc, s->iscal + g.sc + 1);
+                                                                         g.len(), s->iscal + g.sc, s->iscal + g.sc + 1);
         s->launches++;
         if (!sim_cuda_ok(s, cudaGetLastError(), "Galerkin") || !read_scalars(s, u)) return -1;
         W = u[g.sc];
@@ -2012,7 +2139,7 @@ static int resolve_galerkin(sim_t *s, GalerkinJob &g, const int (&v)[kScCount], 
 }
 static Mat<double> job_mat(sim_t *s, const GalerkinJob &g) {
     Mat<double> A;
-    A.st = false; A.selfpad = false; A.diff = false; A.g = s->gd; A.n = g.nc; A.width = g.Wcap; A.col = g.col; A.val = g.val;
+    A.st = false; A.selfpad = false; A.diff = false; A.g = s->gd; A.n = g.nc; A.width = g.Wcap; A.col = g.col; A.val = g.val; A.len = g.len();
     A.wp = s->iscal + g.sc;
     return A;
 }
@@ -2116,7 +2243,7 @@ static sim_status amg_setup(sim_t *s) {
         if (!jm.on) return true;
         const int W = resolve_galerkin(s, jm, v, &rebuilt);
         AmgLevel &L = s->lev.back();
-        L.col = jm.col; L.val = jm.val; L.width = W;
+        L.col = jm.col; L.val = jm.val; L.len = jm.len(); L.width = W;
         dev_free_async(s, old_col); dev_free_async(s, old_val);      // after a rebuild in stream order
         old_col = nullptr; old_val = nullptr;
         if (W < 0) return false;
@@ -2172,7 +2299,7 @@ static sim_status amg_setup(sim_t *s) {
         if (!enqueue_galerkin(s, jm, A1, s->aggB, s->moffB, s->memB, n2, kScM)) return s->err;
         old_col = j1.col; old_val = j1.val;
         AmgLevel C;
-        C.n = n2; C.width = jm.Wcap; C.col = jm.col; C.val = jm.val;
+        C.n = n2; C.width = jm.Wcap; C.col = jm.col; C.val = jm.val; C.len = jm.len();
         s->lev.push_back(C);
     }
     if (jm.on && (!read_scalars(s, v) || !settle(&gone))) return s->err;
@@ -2241,12 +2368,15 @@ sim_status cpr_setup(sim_t *s) {
     return SIM_OK;
 }
 
+// blocks of a launch over the rows of level l (lanes per row on the ELL levels)
+static int level_blocks(int n, int l, int threads) { return sim_blocks((long)n * (l > 0 ? ell_lanes(n) : 1), threads); }
+
 // first level handled by the one-launch coarse cycle (nl: no fusion)
 static int coarse_start(const sim_t *s) {
     const int nl = (int)s->lev.size();
     if (nl < 3) return nl;
     int l0 = nl - 1;
-    while (l0 - 1 >= 1 && s->lev[l0 - 1].n <= kCoarseRows && nl - (l0 - 1) <= kCoarseMaxLevels) l0--;
+    while (l0 - 1 >= 1 && s->lev[l0 - 1].n <= coarse_rows(sim_mixed(s)) && nl - (l0 - 1) <= kCoarseMaxLevels) l0--;
     return (nl - l0 >= 3) ? l0 : nl;   // worth a launch only when it replaces several
 }
 
@@ -2271,21 +2401,61 @@ static L2Prefetch coarse_prefetch(const sim_t *s) {
     return pf;
 }
 
+// a launch of `clusters` clusters of 16 CTAs of kCoarseThreads, or of 8 where an
+// occupancy query finds no room for 16 (a non-portable size); the query launches nothing
+template <typename... KArgs>
+static int coarse_ctas(void (*kernel)(KArgs...)) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 8;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 16; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(16); cfg.blockDim = dim3(kCoarseThreads);
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 8;
+    }
+    return n > 0 ? 16 : 8;
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_clusters(void (*kernel)(KArgs...), int clusters, cudaStream_t st, Args &&...args) {
+    static const int ctas = coarse_ctas(kernel);      // one per kernel (per instantiation of its type)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(clusters * ctas); cfg.blockDim = dim3(kCoarseThreads); cfg.stream = st;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename T>
+static CoarseLevel<T> coarse_level(const AmgLevel &L, int l) {
+    CoarseLevel<T> d;
+    d.n = L.n; d.width = L.width; d.diff = sizeof(T) == sizeof(float); d.st = l == 0; d.colA = L.colA; d.len = L.len; d.val = (const T *)L.valT;
+    d.dinv = (const T *)L.dinvT;
+    d.agg = L.agg; d.moff = L.moff; d.mem = L.mem;
+    d.f = (T *)L.f; d.e = (T *)L.e; d.e2 = (T *)L.e2;
+    return d;
+}
+
 template <typename T>
 static sim_status coarse_cycle(sim_t *s, int l0, const int *done) {
     const int nl = (int)s->lev.size();
     CoarseCycle<T> cc;
-    cc.nlev = nl - l0;
+    cc.nlev = nl - l0; cc.g = s->gd;
     cc.inv = (const double *)s->lev[nl - 1].coarse_inv;
     for (int l = l0; l < nl; l++) {
         const AmgLevel &L = s->lev[l];
         CoarseLevel<T> &d = cc.lv[l - l0];
-        d.n = L.n; d.width = L.width; d.diff = sizeof(T) == sizeof(float); d.colA = L.colA; d.val = (const T *)L.valT;
-        d.dinv = (const T *)L.dinvT;
-        d.agg = L.agg; d.moff = L.moff; d.mem = L.mem;
-        d.f = (T *)L.f; d.e = (T *)L.e; d.e2 = (T *)L.e2;
+        d = coarse_level<T>(L, l);
     }
-    coarse_cycle_kernel<T><<<kCoarseCtas, kCoarseThreads, 0, s->stream>>>(cc, done);
+    if (!sim_cuda_ok(s, launch_clusters(coarse_cycle_kernel<T>, 1, s->stream, cc, done), "coarse cycle")) return s->err;
     SIM_LAUNCHED(s);
     return SIM_OK;
 }
@@ -2298,7 +2468,7 @@ static sim_status vcycle(sim_t *s, const int *done) {
     for (int l = 0; l + 1 < nl && l < lf; l++) {
         AmgLevel &L = s->lev[l], &C = s->lev[l + 1];
         const bool coarsest = (l + 1 == nl - 1);
-        amg_resid_kernel<T><<<sim_blocks(L.n, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
+        amg_resid_kernel<T><<<level_blocks(L.n, l, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
                                                                         (const T *)L.e, (T *)L.e2, done);
         SIM_LAUNCHED(s);
         amg_restrict_kernel<T><<<sim_blocks(C.n, s->tune_amg), s->tune_amg, 0, s->stream>>>((const T *)L.e2, L.moff, L.mem, C.n, (T *)C.f,
@@ -2320,7 +2490,7 @@ static sim_status vcycle(sim_t *s, const int *done) {
         const T *ec = (l + 1 == nl - 1) ? (const T *)C.e : (const T *)C.e2;
         amg_prolong_kernel<T><<<sim_blocks(L.n, s->tune_amg), s->tune_amg, 0, s->stream>>>(L.n, L.agg, ec, (T *)L.e, done);
         SIM_LAUNCHED(s);
-        amg_smooth_kernel<T><<<sim_blocks(L.n, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
+        amg_smooth_kernel<T><<<level_blocks(L.n, l, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
                                                                          (const T *)L.e, (const T *)L.dinvT, (T *)L.e2,
                                                                          done);
         SIM_LAUNCHED(s);
@@ -2507,7 +2677,7 @@ __global__ void b_amg_down_kernel(const CMember<T> *M, const int2 *work, int l, 
     const int i = vb * blockDim.x + threadIdx.x;
     const BLevel<T> &L = m.lv[l];
     if (mode == 0) {
-        if (i < L.n) L.e2[i] = L.f[i] - row_dot(L.A, i, L.e);
+        amg_resid_row<T>(L.A, L.f, L.e, L.e2, i);
     } else {
         const BLevel<T> &C = m.lv[l + 1];
         if (i < C.n) amg_restrict_row<T>(L.e2, L.moff, L.mem, C.f, l + 1 == m.nl - 1 ? nullptr : C.e, C.dinv, i);
@@ -2522,13 +2692,13 @@ __global__ void b_amg_up_kernel(const CMember<T> *M, const int2 *work, int l, in
     if (skip(m.done)) return;
     const int i = vb * blockDim.x + threadIdx.x;
     const BLevel<T> &L = m.lv[l];
-    if (i >= L.n) return;
     if (mode == 0) {
+        if (i >= L.n) return;
         const BLevel<T> &C = m.lv[l + 1];
         const T *ec = (l + 1 == m.nl - 1) ? C.e : C.e2;
         L.e[i] += ec[L.agg[i]];
     } else {
-        L.e2[i] = L.e[i] + (L.f[i] - row_dot(L.A, i, L.e)) * L.dinv[i];
+        amg_smooth_row<T>(L.A, L.f, L.e, L.dinv, L.e2, i);
     }
 }
 
@@ -2550,11 +2720,11 @@ __global__ void b_coarse_solve_kernel(const CMember<T> *M, const int2 *work) {
 
 // the fused coarse levels: cluster c runs member members[c]
 template <typename T>
-__global__ void __cluster_dims__(kCoarseCtas, 1, 1) __launch_bounds__(kCoarseThreads, 1)
-b_coarse_cycle_kernel(const CMember<T> *M, const int *members) {
-    const CMember<T> &m = M[members[blockIdx.x / kCoarseCtas]];
+__global__ void __launch_bounds__(kCoarseThreads, 1) b_coarse_cycle_kernel(const CMember<T> *M, const int *members) {
+    const int nb = (int)cg::this_cluster().num_blocks();
+    const CMember<T> &m = M[members[blockIdx.x / nb]];
     if (skip(m.done)) return;          // uniform over the cluster (one member)
-    coarse_cycle_body<T>(*m.cc, (int)(blockIdx.x % kCoarseCtas), kCoarseCtas);
+    coarse_cycle_body<T>(*m.cc, (int)(blockIdx.x % nb), nb);
 }
 
 // stage F on the residual of stage P: sweep 0 (all cells), 1 (black), 2 (red,
@@ -2589,7 +2759,7 @@ struct CprBatch {
     int ncl = 0;
     struct List { long off = 0; int count = 0; };
     List cell256, cell64, stage1, stage2, cs;
-    std::vector<List> down_r, down_c, up;
+    std::vector<List> down_r, down_c, up, up_s;
 };
 
 static cudaError_t grow(void **p, size_t *cap, size_t bytes) {
@@ -2624,7 +2794,7 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
     std::vector<CoarseCycle<T>> hcc;
     std::vector<int> hcl;
     std::vector<int2> work;
-    cb->down_r.clear(); cb->down_c.clear(); cb->up.clear();
+    cb->down_r.clear(); cb->down_c.clear(); cb->up.clear(); cb->up_s.clear();
     auto add_list = [&](CprBatch::List &L, auto blocks_of) {
         L.off = (long)work.size();
         for (int k = 0; k < nm; k++) {
@@ -2662,15 +2832,12 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
         }
         if (m.lf < nl) {
             CoarseCycle<T> cc;
-            cc.nlev = nl - m.lf;
+            cc.nlev = nl - m.lf; cc.g = s->gd;
             cc.inv = m.inv;
             for (int l = m.lf; l < nl; l++) {
                 const AmgLevel &L = s->lev[l];
                 CoarseLevel<T> &d = cc.lv[l - m.lf];
-                d.n = L.n; d.width = L.width; d.diff = sizeof(T) == sizeof(float); d.colA = L.colA;
-                d.val = (const T *)L.valT; d.dinv = (const T *)L.dinvT;
-                d.agg = L.agg; d.moff = L.moff; d.mem = L.mem;
-                d.f = (T *)L.f; d.e = (T *)L.e; d.e2 = (T *)L.e2;
+                d = coarse_level<T>(L, l);
             }
             hcc.push_back(cc);
             hcl.push_back(k);
@@ -2688,13 +2855,15 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
     add_list(cb->stage2, [&](int k) { return hm[k].rb ? colour_blocks(ms[k], kStageThreads) : sim_blocks(hm[k].g.N, kStageThreads); });
     add_list(cb->cs, [&](int k) { const CMember<T> &m = hm[k];
                                   return (m.nl == 1 || m.lf == m.nl) ? sim_blocks((long)m.lv[m.nl - 1].n * 32, SIM_THREADS) : 0; });
-    cb->down_r.resize(maxdown); cb->down_c.resize(maxdown); cb->up.resize(maxup);
+    cb->down_r.resize(maxdown); cb->down_c.resize(maxdown); cb->up.resize(maxup); cb->up_s.resize(maxup);
     for (int l = 0; l < maxdown; l++) {
-        add_list(cb->down_r[l], [&](int k) { return l < down_of(k) ? sim_blocks(hm[k].lv[l].n, kBatchAmgThreads) : 0; });
+        add_list(cb->down_r[l], [&](int k) { return l < down_of(k) ? level_blocks(hm[k].lv[l].n, l, kBatchAmgThreads) : 0; });
         add_list(cb->down_c[l], [&](int k) { return l < down_of(k) ? sim_blocks(hm[k].lv[l + 1].n, kBatchAmgThreads) : 0; });
     }
-    for (int l = 0; l < maxup; l++)
+    for (int l = 0; l < maxup; l++) {
         add_list(cb->up[l], [&](int k) { return l < top_of(k) ? sim_blocks(hm[k].lv[l].n, kBatchAmgThreads) : 0; });
+        add_list(cb->up_s[l], [&](int k) { return l < top_of(k) ? level_blocks(hm[k].lv[l].n, l, kBatchAmgThreads) : 0; });
+    }
     cudaError_t e;
     if ((e = grow(&cb->dmem, &cb->mem_cap, sizeof(CMember<T>) * nm)) != cudaSuccess) return e;
     if ((e = grow((void **)&cb->dwork, &cb->work_cap, sizeof(int2) * std::max<size_t>(1, work.size()))) != cudaSuccess) return e;
@@ -2743,13 +2912,13 @@ static int batch_apply_t(const CprBatch *cb, cudaStream_t st, int j) {
         go(cb->down_c[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_down_kernel<T><<<n, t, 0, st>>>(M, w, (int)l, 1); });
     }
     if (cb->ncl > 0) {
-        b_coarse_cycle_kernel<T><<<cb->ncl * kCoarseCtas, kCoarseThreads, 0, st>>>(M, cb->dcl);
+        if (launch_clusters(b_coarse_cycle_kernel<T>, cb->ncl, st, M, (const int *)cb->dcl) != cudaSuccess) return -1;
         launches++;
     }
     go(cb->cs, SIM_THREADS, [&](int n, int t, const int2 *w) { b_coarse_solve_kernel<T><<<n, t, 0, st>>>(M, w); });
     for (int l = (int)cb->up.size() - 1; l >= 0; l--) {
         go(cb->up[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_up_kernel<T><<<n, t, 0, st>>>(M, w, l, 0); });
-        go(cb->up[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_up_kernel<T><<<n, t, 0, st>>>(M, w, l, 1); });
+        go(cb->up_s[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_up_kernel<T><<<n, t, 0, st>>>(M, w, l, 1); });
     }
     go(cb->cell64, kStageThreads, [&](int n, int t, const int2 *w) { b_stage2_kernel<B, T><<<n, t, 0, st>>>(M, w, j, 0); });
     go(cb->stage1, kStageThreads, [&](int n, int t, const int2 *w) { b_stage2_kernel<B, T><<<n, t, 0, st>>>(M, w, j, 1); });

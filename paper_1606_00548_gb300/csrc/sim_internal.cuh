@@ -108,6 +108,7 @@ struct BicgCtl {
 struct AmgLevel {
     int n = 0, width = 0;        // level 0: width 7, structured
     int *col = nullptr;          // ELL columns [width][n] (levels >= 1), -1 padding
+    int *len = nullptr;          // entries of each row (behind col in its allocation)
     int *colA = nullptr;         // the same with padding on the row's own column (apply)
     double *val = nullptr;       // ELL values, FP64 (setup precision)
     void *valT = nullptr;        // ELL values in apply precision (float copy for mixed)
