@@ -40,7 +40,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-__device__ __forceinline__ uint32_t bf16_bits(const uint16_t *p) { return (uint32_t)(*p); }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {
@@ -241,6 +240,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
                                                                 const int *done, int *__restrict__ status,
                                                                 int stall_slab) {
     if (done != nullptr && *(volatile const int *)done) return;
+    // The next layer's convolution may start as this one's CTAs leave their SMs: what
+    // it does before its own wait (barriers, weights, tensor memory) reads nothing this
+    // kernel writes, and the wait below returns when the kernel before has completed
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ uint8_t tc_raw[];
     __shared__ TcBars bars;
     __shared__ uint32_t tmem_base;
@@ -276,6 +279,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = tmem_base;
@@ -445,17 +449,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
 // weight gradient: dW[t][ci][co] = sum over cells c of In[c + off(t)][ci] * G[c][co]
 // (mma.sync.m16n8k16 BF16 -> FP32; per tap a 16 x 16 product with the cells
 // as the contraction: too narrow for the 128-row tcgen05 tile).
-// Persistent, two CTAs per SM, bricks of 128 x 1 x WG_TZ cells dealt
-// round-robin.  Per brick one thread stages by TMA the three input slabs
-// (y-1, y, y+1; lines z0-1 .. z0+WG_TZ; cells x0-8 .. x0+135) and the brick's
-// output-gradient lines, both activation planes each, in the rows of 16 bytes
-// the activations have; out-of-grid cells arrive as zeros (bounds fill and x
-// padding), so no cell is masked.  Warp w owns taps w, w+8, w+16, w+24; per
+// Persistent, two CTAs per SM, bricks of 128 x 1 x WG_TZ cells in runs of up to
+// WG_RUN along y, dealt round-robin, the runs of a ragged last x column after all
+// others.  One thread stages by TMA the brick's input slabs (y-1, y, y+1; lines
+// z0-1 .. z0+WG_TZ; cells x0-8 .. x0+135) and its output-gradient lines, both
+// activation planes each, in the rows of 16 bytes the activations have; a run keeps
+// its slabs in a ring of three and stages one new slab a brick (44 KB of L2 reads
+// instead of 99).  Bound by the legacy tensor path: about 24 clocks per MMA and
+// sub-partition, 27 us for 131 x 67 x 29 cells (28 us with three slabs a brick).
+// Out-of-grid cells arrive as zeros (bounds fill and x padding), so no cell is masked.  Warp w owns taps w, w+8, w+16, w+24; per
 // 16-cell step it loads the gradient fragment once (ldmatrix.trans: rows are
 // cells) and, per tap, the input fragment of the shifted cells, and issues two
-// MMAs (output channels 0-7, 8-15).  Accumulators stay in registers across the
-// CTA's bricks; each CTA writes one partial [27][16][16], folded in CTA order
-// (deterministic).  Waits are bounded (status bit 4 on a timeout).
+// MMAs (output channels 0-7, 8-15; the second not where the layer has at most eight
+// outputs, nor any past the last 16-cell step of a ragged x).  Warp 3's fourth slot
+// is a 28th tap whose input is one everywhere: its product is the bias gradient.
+// Accumulators stay in registers across the CTA's bricks; each CTA writes one partial
+// [28][16][16], folded in a fixed order.  Waits are bounded (status bit 4 on a timeout).
 // ---------------------------------------------------------------------------
 constexpr int WG_TZ = 4;                                   // output lines per brick (z)
 constexpr int WG_SZ = WG_TZ + 2;                           // staged lines per input slab
@@ -464,6 +473,7 @@ constexpr int WG_GBOX = WG_TZ * TC_M * 16;                 // output-gradient li
 constexpr int WG_IN = 6 * WG_IBOX;                         // 3 slabs x 2 planes
 constexpr int WG_SMEM = WG_IN + 2 * WG_GBOX + 128;
 constexpr int WG_THREADS = 256;
+constexpr int WG_TAPS = 28;                                // 27 and the bias
 static_assert(WG_IBOX % 128 == 0 && WG_GBOX % 128 == 0, "TMA destinations 128-byte aligned");
 static_assert(2 * (WG_SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
 
@@ -475,7 +485,7 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t 
 
 __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_constant__ CUtensorMap tin,
                                                                  const __grid_constant__ CUtensorMap tg, Dims d,
-                                                                 int nbricks, float *__restrict__ part,
+                                                                 int run, int cout, float *__restrict__ part,
                                                                  int *__restrict__ status) {
     extern __shared__ uint8_t wg_raw[];
     __shared__ uint64_t bar;
@@ -484,7 +494,8 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
     uint8_t *sin = wg_raw + ((128u - (smem_addr(wg_raw) & 127u)) & 127u);
     uint8_t *sg = sin + WG_IN;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int gx = (d.nx + TC_M - 1) / TC_M;
+    const int gz = (d.nz + WG_TZ - 1) / WG_TZ, gy = (d.ny + run - 1) / run;
+    const int nruns = ((d.nx + TC_M - 1) / TC_M) * gy * gz;
     if (tid == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -504,53 +515,71 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
     const uint32_t s_in = smem_addr(sin), s_g = smem_addr(sg);
     int it = 0;
     bool in_flight = false;   // thread 0: the current brick's copies were started and not yet waited for
-    for (int br = blockIdx.x; br < nbricks && !*abort; br += gridDim.x, it++) {
-        const int bx = br % gx, r = br / gx, y = r % d.ny, bz = r / d.ny;
-        const int x0 = bx * TC_M, z0 = bz * WG_TZ;
-        if (tid == 0) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_expect(&bar, WG_IN + 2 * WG_GBOX);
-            for (int s = 0; s < 3; s++)
-                for (int h = 0; h < 2; h++)
-                    tma_load_5d(sin + (s * 2 + h) * WG_IBOX, &tin, 0, x0 / 8 - 1, y - 1 + s, z0 - 1, h, &bar);
-            for (int h = 0; h < 2; h++) tma_load_5d(sg + h * WG_GBOX, &tg, 0, x0 / 8, y, z0, h, &bar);
-            in_flight = true;
-        }
-        const bool ok = mbar_wait(&bar, it & 1, abort, status, 16);
-        if (tid == 0 && ok) in_flight = false;
-        if (__syncthreads_or(!ok)) break;   // every thread leaves together: no barrier below waits on one that left
-        for (int zo = 0; zo < WG_TZ; zo++) {
-            for (int xk = 0; xk < TC_M; xk += 16) {
-                // gradient fragment (B, 16 cells x 16 outputs): matrices (plane 0, cells 0-7), (0, 8-15), (1, 0-7), (1, 8-15)
-                uint32_t b[4];
-                ldsm_x4_t(s_g + (uint32_t)((mat >> 1) * WG_GBOX + ((zo * TC_M + xk + (mat & 1) * 8 + mrow) * 16)), b[0], b[1],
-                          b[2], b[3]);
+    // tap t of this warp's slot j: where its input fragment of the brick's first cells
+    // lies in a slab (matrices (plane 0, cells 0-7), (1, 0-7), (0, 8-15), (1, 8-15) at
+    // the shifted cells), and the slab (0: y - 1)
+    uint32_t a_off[4];
+    int a_slab[4];
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const int t = warp + 8 * j;
-                    if (t < 27) {
-                        const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-                        // input fragment (A, 16 channels x 16 cells) at the shifted cells:
-                        // matrices (plane 0, cells 0-7), (1, 0-7), (0, 8-15), (1, 8-15)
-                        const int cell = (zo + dz + 1) * TC_XS + xk + dx + 8 + (mat >> 1) * 8 + mrow;
+    for (int j = 0; j < 4; j++) {
+        const int t = warp + 8 * j, dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
+        a_slab[j] = dy + 1;
+        a_off[j] = s_in + (uint32_t)((mat & 1) * WG_IBOX + ((dz + 1) * TC_XS + dx + 8 + (mat >> 1) * 8 + mrow) * 16);
+    }
+    const uint32_t g_off = s_g + (uint32_t)((mat >> 1) * WG_GBOX + ((mat & 1) * 8 + mrow) * 16);
+    bool stop = false;
+    for (int c = blockIdx.x; c < nruns && !stop && !*abort; c += gridDim.x) {
+        const int yc = c % gy, bz = (c / gy) % gz, bx = c / (gy * gz);
+        const int x0 = bx * TC_M, z0 = bz * WG_TZ, ya = yc * run, yb = min(d.ny, ya + run);
+        const int xend = min(TC_M, d.nx - x0), zend = min(WG_TZ, d.nz - z0);   // beyond: zero gradients
+        for (int y = ya; y < yb; y++, it++) {
+            if (tid == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                const int s0 = y == ya ? 0 : 2;          // slabs y-1+s0 .. y+1 are new; slab y' lies in slot (y' + 1) mod 3
+                mbar_expect(&bar, (3 - s0) * 2 * WG_IBOX + 2 * WG_GBOX);
+                for (int s = s0; s < 3; s++)
+                    for (int h = 0; h < 2; h++)
+                        tma_load_5d(sin + (((y + s) % 3) * 2 + h) * WG_IBOX, &tin, 0, x0 / 8 - 1, y - 1 + s, z0 - 1, h, &bar);
+                for (int h = 0; h < 2; h++) tma_load_5d(sg + h * WG_GBOX, &tg, 0, x0 / 8, y, z0, h, &bar);
+                in_flight = true;
+            }
+            const bool ok = mbar_wait(&bar, it & 1, abort, status, 16);
+            if (tid == 0 && ok) in_flight = false;
+            stop = __syncthreads_or(!ok) != 0;
+            if (stop) break;   // every thread leaves together: no barrier below waits on one that left
+            uint32_t abase[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) abase[j] = a_off[j] + (uint32_t)((y + a_slab[j]) % 3) * (2 * WG_IBOX);
+            for (int zo = 0; zo < zend; zo++) {
+                for (int xk = 0; xk < xend; xk += 16) {
+                    // gradient fragment (B, 16 cells x 16 outputs): matrices (plane 0, cells 0-7), (0, 8-15), (1, 0-7), (1, 8-15)
+                    uint32_t b[4];
+                    ldsm_x4_t(g_off + (uint32_t)((zo * TC_M + xk) * 16), b[0], b[1], b[2], b[3]);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int t = warp + 8 * j;
+                        if (t >= WG_TAPS) continue;
                         uint32_t a[4];
-                        ldsm_x4_t(s_in + (uint32_t)(((dy + 1) * 2 + (mat & 1)) * WG_IBOX + cell * 16), a[0], a[1], a[2], a[3]);
+                        if (t < 27)
+                            ldsm_x4_t(abase[j] + (uint32_t)((zo * TC_XS + xk) * 16), a[0], a[1], a[2], a[3]);
+                        else
+                            a[0] = a[1] = a[2] = a[3] = 0x3f803f80u;   // BF16 ones
                         mma_bf16(acc[j][0], a[0], a[1], a[2], a[3], b[0], b[1]);
-                        mma_bf16(acc[j][1], a[0], a[1], a[2], a[3], b[2], b[3]);
+                        if (cout > 8) mma_bf16(acc[j][1], a[0], a[1], a[2], a[3], b[2], b[3]);
                     }
                 }
             }
+            __syncthreads();   // every warp is done with the buffers before the next brick's copies
         }
-        __syncthreads();   // every warp is done with the buffers before the next brick's copies
     }
     if (tid == 0 && in_flight && !mbar_drain(&bar, it & 1)) atomicOr(status, 16);
-    // partial of this CTA: [27][16 ci][16 co]
+    // partial of this CTA: [28][16 ci][16 co]
     const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
         const int t = warp + 8 * j;
-        if (t >= 27) continue;
-        float *o = part + ((long)blockIdx.x * 27 + t) * 256;
+        if (t >= WG_TAPS) continue;
+        float *o = part + ((long)blockIdx.x * WG_TAPS + t) * 256;
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int co = 8 * h + 2 * t4;
@@ -562,45 +591,41 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
     }
 }
 
-// dW[t][ci][co] (FP32, logical cin x cout) = sum of the CTAs' partials, in CTA order
-__global__ void wgrad_fold_kernel(int nblk, int cin, int cout, const float *__restrict__ part, float *__restrict__ dW) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= 27 * cin * cout) return;
-    const int tap = e / (cin * cout), r = e % (cin * cout), ci = r / cout, co = r % cout;
-    float s = 0.f;
-    for (int b = 0; b < nblk; b++) s += part[((long)b * 27 + tap) * 256 + ci * 16 + co];
-    dW[e] = s;
-}
-
-// bias gradient partials: per block sums of dout channels
-__global__ void bgrad_kernel(Dims d, int cout, const uint16_t *__restrict__ dout, float *__restrict__ part) {
-    __shared__ float sh[128][16];
-    float s[16];
-    for (int c = 0; c < 16; c++) s[c] = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.N; i += gridDim.x * blockDim.x)
-        for (int c = 0; c < cout; c++) s[c] += __uint_as_float(bf16_bits(dout + act_elem_c(d, i, c)) << 16);
-    for (int c = 0; c < 16; c++) sh[threadIdx.x][c] = s[c];
+// dW[t][ci][co] (FP32, logical cin x cout) and, behind it, db[co] = sums of the CTAs'
+// partials in a fixed order: eight threads per entry take every eighth CTA, then add
+// up (one thread per entry waited on 304 loads in turn: 18 us, now 4 us)
+__global__ void __launch_bounds__(256) wgrad_fold_kernel(int nblk, int cin, int cout, const float *__restrict__ part,
+                                                         float *__restrict__ dW) {
+    __shared__ float sh[8][32];
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane, nw = 27 * cin * cout;
+    if (e < nw + cout) {
+        const int tap = e < nw ? e / (cin * cout) : 27, r = e < nw ? e % (cin * cout) : e - nw;
+        const float *p = part + (long)tap * 256 + (r / cout) * 16 + r % cout;
+        float s = 0.f;
+#pragma unroll 8
+        for (int b = seg; b < nblk; b += 8) s += p[(long)b * WG_TAPS * 256];
+        sh[seg][lane] = s;
+    }
     __syncthreads();
-    if (threadIdx.x < 16) {
-        float t = 0.f;
-        for (int k = 0; k < (int)blockDim.x; k++) t += sh[k][threadIdx.x];
-        part[blockIdx.x * 16 + threadIdx.x] = t;
+    if (seg == 0 && e < nw + cout) {
+        float s = sh[0][lane];
+#pragma unroll
+        for (int q = 1; q < 8; q++) s += sh[q][lane];
+        dW[e] = s;
     }
 }
-__global__ void bgrad_fold_kernel(int nblk, int cout, const float *__restrict__ part, float *__restrict__ db) {
-    const int c = threadIdx.x;
-    if (c >= cout) return;
-    float t = 0.f;
-    for (int b = 0; b < nblk; b++) t += part[b * 16 + c];
-    db[c] = t;
-}
 
-// MSE loss partials and dL/dy = 2 (y - target) / N into channel 0 of a planar BF16 buffer
-__global__ void mse_kernel(Dims d, const float *__restrict__ y, const float *__restrict__ target, uint16_t *__restrict__ dout,
-                           double *__restrict__ part) {
-    __shared__ double sh[128];
+// MSE loss and dL/dy = 2 (y - target) / N into channel 0 of a planar BF16 buffer; the
+// last block to finish adds the per-block partials in block order
+constexpr int kLossBlocks = 608;
+__global__ void __launch_bounds__(256) mse_kernel(Dims d, const float *__restrict__ y, const float *__restrict__ target,
+                                                  uint16_t *__restrict__ dout, double *__restrict__ part,
+                                                  unsigned int *ticket, double *__restrict__ loss) {
+    __shared__ double sh[8];
+    __shared__ bool last;
     double s = 0.0;
-    const int N = d.N;
+    const int N = d.N, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const float scale = 2.0f / (float)N;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         const float e = y[i] - target[i];
@@ -609,19 +634,23 @@ __global__ void mse_kernel(Dims d, const float *__restrict__ y, const float *__r
         *o0 = make_uint4(pack_bf16(e * scale, 0.f), 0u, 0u, 0u);
         *o1 = make_uint4(0u, 0u, 0u, 0u);
     }
-    sh[threadIdx.x] = s;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) sh[wid] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int k = 0; k < (int)blockDim.x; k++) t += sh[k];
+        for (int k = 0; k < 8; k++) t += sh[k];
         part[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-}
-__global__ void mse_fold_kernel(int nblk, int N, const double *__restrict__ part, double *__restrict__ loss) {
-    if (threadIdx.x != 0) return;
+    __syncthreads();
+    if (!last || wid != 0) return;
+    __threadfence();
     double t = 0.0;
-    for (int b = 0; b < nblk; b++) t += part[b];
-    *loss = t / N;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + b);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) { *loss = t / N; *ticket = 0u; }
 }
 
 // FP32 features [N][4] -> planar BF16 activations (channels 4..15 zero)
@@ -689,9 +718,14 @@ struct sim_net {
     int stall_once = -1;                 // testing hook: slab whose copy the next forward pass skips
     float *out = nullptr;                // [N]
     uint32_t *g0 = nullptr, *g1 = nullptr;   // BF16 [N][16] gradient buffers
-    float *wpart = nullptr, *bpart = nullptr;
+    float *wpart = nullptr;
     double *lpart = nullptr, *dloss = nullptr;
-    int wg_ctas = 0, bblk = 0, lblk = 0;
+    unsigned int *lticket = nullptr;     // last-block ticket of the loss
+    // what a call returns to the host lies together on the device (gradients, loss,
+    // ticket, status word) and comes back in one copy into pinned memory
+    size_t ret_bytes = 0, ret_loss = 0, ret_stat = 0;
+    char *hret = nullptr;
+    int wg_ctas = 0, lblk = 0;
     int adam_t = 0;
     int64_t launches = 0;
 };
@@ -710,12 +744,16 @@ static bool net_ok(sim_net_t *n, cudaError_t e, const char *what) {
 
 // the convolutions' status word, read after the stream has drained: non-zero
 // means a bounded wait inside a convolution gave up (its output was skipped)
-static sim_status net_status(sim_net_t *n) {
+static sim_status net_status_value(sim_net_t *n) {
     int st = 0;
-    NET_CK(n, cudaMemcpyAsync(&st, n->dstat, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
-    NET_CK(n, cudaStreamSynchronize(n->stream));
+    memcpy(&st, n->hret + n->ret_stat, sizeof(int));
     if (st != 0) return net_fail(n, SIM_ETIMEOUT, "convolution: a bounded wait gave up (status " + std::to_string(st) + ")");
     return SIM_OK;
+}
+static sim_status net_status(sim_net_t *n) {
+    NET_CK(n, cudaMemcpyAsync(n->hret + n->ret_stat, n->dstat, sizeof(int), cudaMemcpyDeviceToHost, n->stream));
+    NET_CK(n, cudaStreamSynchronize(n->stream));
+    return net_status_value(n);
 }
 
 static void *net_alloc(sim_net_t *n, size_t bytes) {
@@ -788,10 +826,16 @@ static int tc_grid(const Dims &d) {
     return nb < sms ? nb : sms;
 }
 
-static int wg_bricks(const Dims &d) { return ((d.nx + TC_M - 1) / TC_M) * d.ny * ((d.nz + WG_TZ - 1) / WG_TZ); }
-// persistent weight-gradient grid: two CTAs per SM, at most one per brick
+// weight gradient: the longest run of bricks along y that still gives every CTA one,
+// and the persistent grid, two CTAs per SM, at most one per run
+constexpr int WG_RUN = 8;
+static int wg_columns(const Dims &d) { return ((d.nx + TC_M - 1) / TC_M) * ((d.nz + WG_TZ - 1) / WG_TZ); }
+static int wg_run(const Dims &d) {
+    const int r = (int)((long)wg_columns(d) * d.ny / (2 * tc_grid_sms()));
+    return r < 1 ? 1 : r < WG_RUN ? r : WG_RUN;
+}
 static int wg_grid(const Dims &d) {
-    const int nb = wg_bricks(d), two = 2 * tc_grid_sms();
+    const int run = wg_run(d), nb = wg_columns(d) * ((d.ny + run - 1) / run), two = 2 * tc_grid_sms();
     return nb < two ? nb : two;
 }
 
@@ -806,20 +850,28 @@ static bool tc_attrs() {
     return ok;
 }
 
-static sim_status net_forward(sim_net_t *n, const int *done = nullptr) {
+// the four layers from act[0] into outf
+static sim_status net_forward(sim_net_t *n, float *outf, const int *done = nullptr) {
     if (!tc_attrs()) return net_fail(n, SIM_ECUDA, "convolution kernel attributes");
     const int grid = tc_grid(n->d), nb = tc_bricks(n->d);
     const int stall = n->stall_once;
     n->stall_once = -1;
     for (int l = 0; l < NLAYER; l++) {
         const float *bias = n->param + n->off_b[l];
-        if (l + 1 < NLAYER)
-            conv_tc_kernel<0><<<grid, TC_THREADS, TC_SMEM, n->stream>>>(n->map_act[l], n->d, nb, n->wf[l], bias, nullptr,
-                                                                        n->act[l + 1], nullptr, done, n->dstat,
-                                                                        l == 0 ? stall : -1);
-        else
-            conv_tc_kernel<1><<<grid, TC_THREADS, TC_SMEM, n->stream>>>(n->map_act[l], n->d, nb, n->wf[l], bias, nullptr,
-                                                                        nullptr, n->out, done, n->dstat, -1);
+        const bool last = l + 1 == NLAYER;
+        // layers after the first overlap their prologue with the one before (524k cells:
+        // 94 us a forward pass, 107 without); not inside a solver's captured cycle
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = TC_SMEM; cfg.stream = n->stream;
+        cfg.attrs = at; cfg.numAttrs = l > 0 && done == nullptr ? 1 : 0;
+        const cudaError_t e = cudaLaunchKernelEx(
+            &cfg, last ? conv_tc_kernel<1> : conv_tc_kernel<0>, n->map_act[l], n->d, nb, (const uint16_t *)n->wf[l], bias,
+            (const uint32_t *)nullptr, last ? (uint32_t *)nullptr : n->act[l + 1], last ? outf : (float *)nullptr, done,
+            n->dstat, l == 0 ? stall : -1);
+        if (!net_ok(n, e, "convolution launch")) return n->err;
         NET_LAUNCHED(n);
     }
     return SIM_OK;
@@ -827,25 +879,17 @@ static sim_status net_forward(sim_net_t *n, const int *done = nullptr) {
 
 // gradients of the MSE loss of the last forward pass into n->grad; loss into n->dloss
 static sim_status net_backward(sim_net_t *n, const float *target) {
-    const int N = n->d.N;
-    mse_kernel<<<n->lblk, 128, 0, n->stream>>>(n->d, n->out, target, (uint16_t *)n->g0, n->lpart);
-    NET_LAUNCHED(n);
-    mse_fold_kernel<<<1, 32, 0, n->stream>>>(n->lblk, N, n->lpart, n->dloss);
+    mse_kernel<<<n->lblk, 256, 0, n->stream>>>(n->d, n->out, target, (uint16_t *)n->g0, n->lpart, n->lticket, n->dloss);
     NET_LAUNCHED(n);
     if (!tc_attrs()) return net_fail(n, SIM_ECUDA, "convolution kernel attributes");
     uint32_t *gcur = n->g0, *gnext = n->g1;
     for (int l = NLAYER - 1; l >= 0; l--) {
         const int gi = gcur == n->g0 ? 0 : 1;
-        wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[gi], n->d, wg_bricks(n->d),
-                                                                       n->wpart, n->dstat);
+        wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[gi], n->d, wg_run(n->d),
+                                                                       COUT[l], n->wpart, n->dstat);
         NET_LAUNCHED(n);
-        const int ne = 27 * CIN[l] * COUT[l];
-        wgrad_fold_kernel<<<sim_blocks(ne), SIM_THREADS, 0, n->stream>>>(n->wg_ctas, CIN[l], COUT[l], n->wpart,
-                                                                          n->grad + n->off_w[l]);
-        NET_LAUNCHED(n);
-        bgrad_kernel<<<n->bblk, 128, 0, n->stream>>>(n->d, COUT[l], (const uint16_t *)gcur, n->bpart);
-        NET_LAUNCHED(n);
-        bgrad_fold_kernel<<<1, 32, 0, n->stream>>>(n->bblk, COUT[l], n->bpart, n->grad + n->off_b[l]);
+        wgrad_fold_kernel<<<sim_blocks(27 * CIN[l] * COUT[l] + COUT[l], 32), 256, 0, n->stream>>>(
+            n->wg_ctas, CIN[l], COUT[l], n->wpart, n->grad + n->off_w[l]);
         NET_LAUNCHED(n);
         if (l > 0) {   // data gradient through layer l into the ReLU output of layer l-1
             conv_tc_kernel<2><<<tc_grid(n->d), TC_THREADS, TC_SMEM, n->stream>>>(
@@ -887,7 +931,14 @@ sim_status sim_net_create(int32_t nx, int32_t ny, int32_t nz, uint64_t seed, voi
     bool ok = true;
     auto A = [&](size_t b) -> void * { void *p = ok ? net_alloc(n, b) : nullptr; if (!p) ok = false; return p; };
     n->param = (float *)A(sizeof(float) * off);
-    n->grad = (float *)A(sizeof(float) * off);
+    n->ret_loss = (sizeof(float) * off + 7) & ~(size_t)7;
+    n->ret_stat = n->ret_loss + sizeof(double) + sizeof(unsigned int);
+    n->ret_bytes = n->ret_stat + sizeof(int);
+    char *ret = (char *)A(n->ret_bytes);
+    n->grad = (float *)ret;
+    n->dloss = (double *)(ret + n->ret_loss);
+    n->lticket = (unsigned int *)(ret + n->ret_loss + sizeof(double));
+    n->dstat = (int *)(ret + n->ret_stat);
     n->adam_m = (float *)A(sizeof(float) * off);
     n->adam_v = (float *)A(sizeof(float) * off);
     for (int l = 0; l < NLAYER; l++) {
@@ -900,13 +951,10 @@ sim_status sim_net_create(int32_t nx, int32_t ny, int32_t nz, uint64_t seed, voi
     n->g0 = (uint32_t *)A(act_bytes);
     n->g1 = (uint32_t *)A(act_bytes);
     n->wg_ctas = wg_grid(n->d);
-    n->wpart = (float *)A(sizeof(float) * 27 * 256 * (size_t)n->wg_ctas);
-    n->bblk = 256;
-    n->bpart = (float *)A(sizeof(float) * n->bblk * 16);
-    n->lblk = 256;
-    n->lpart = (double *)A(sizeof(double) * n->lblk);
-    n->dloss = (double *)A(sizeof(double) * 2);
-    n->dstat = (int *)A(sizeof(int));
+    n->wpart = (float *)A(sizeof(float) * WG_TAPS * 256 * (size_t)n->wg_ctas);
+    n->lblk = sim_blocks(N) < kLossBlocks ? sim_blocks(N) : kLossBlocks;
+    n->lpart = (double *)A(sizeof(double) * kLossBlocks);
+    if (ok && cudaMallocHost((void **)&n->hret, n->ret_bytes) != cudaSuccess) { n->hret = nullptr; ok = false; }
     if (!ok) {
         std::string m = n->msg;
         sim_net_destroy(n);
@@ -939,7 +987,7 @@ sim_status sim_net_create(int32_t nx, int32_t ny, int32_t nz, uint64_t seed, voi
     }
     if (cudaMemcpy(n->param, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(n->adam_m, 0, sizeof(float) * off) != cudaSuccess ||
-        cudaMemset(n->adam_v, 0, sizeof(float) * off) != cudaSuccess || cudaMemset(n->dstat, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(n->adam_v, 0, sizeof(float) * off) != cudaSuccess || cudaMemset(n->dloss, 0, n->ret_bytes - n->ret_loss) != cudaSuccess ||
         !zero_acts(n, act_bytes) || pack_all(n) != SIM_OK) {
         sim_net_destroy(n);
         return sim_fail(nullptr, SIM_ECUDA, "sim_net_create: initialisation failed");
@@ -952,6 +1000,7 @@ void sim_net_destroy(sim_net_t *n) {
     if (!n) return;
     if (n->stream) cudaStreamSynchronize(n->stream);
     for (void *p : n->allocs) cudaFree(p);
+    if (n->hret) cudaFreeHost(n->hret);
     if (n->own_stream && n->stream) cudaStreamDestroy(n->stream);
     delete n;
 }
@@ -979,8 +1028,7 @@ sim_status sim_net_forward(sim_net_t *n, const float *x_dev, float *y_dev) {
     if (n->err != SIM_OK) return n->err;
     features_kernel<<<sim_blocks(n->d.N), SIM_THREADS, 0, n->stream>>>(n->d, x_dev, (uint16_t *)n->act[0], nullptr);
     NET_LAUNCHED(n);
-    if (net_forward(n) != SIM_OK) return n->err;
-    NET_CK(n, cudaMemcpyAsync(y_dev, n->out, sizeof(float) * n->d.N, cudaMemcpyDeviceToDevice, n->stream));
+    if (net_forward(n, y_dev) != SIM_OK) return n->err;
     return net_status(n);
 }
 
@@ -989,13 +1037,13 @@ sim_status sim_net_loss_grad(sim_net_t *n, const float *x_dev, const float *targ
     if (n->err != SIM_OK) return n->err;
     features_kernel<<<sim_blocks(n->d.N), SIM_THREADS, 0, n->stream>>>(n->d, x_dev, (uint16_t *)n->act[0], nullptr);
     NET_LAUNCHED(n);
-    if (net_forward(n) != SIM_OK || net_backward(n, target_dev) != SIM_OK) return n->err;
-    double l = 0.0;
-    NET_CK(n, cudaMemcpyAsync(&l, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
-    if (grads) NET_CK(n, cudaMemcpyAsync(grads, n->grad, sizeof(float) * n->nparam, cudaMemcpyDeviceToHost, n->stream));
+    if (net_forward(n, n->out) != SIM_OK || net_backward(n, target_dev) != SIM_OK) return n->err;
+    const size_t from = grads ? 0 : n->ret_loss;
+    NET_CK(n, cudaMemcpyAsync(n->hret + from, (char *)n->grad + from, n->ret_bytes - from, cudaMemcpyDeviceToHost, n->stream));
     NET_CK(n, cudaStreamSynchronize(n->stream));
-    if (loss) *loss = l;
-    return net_status(n);
+    if (grads) memcpy(grads, n->hret, sizeof(float) * n->nparam);
+    if (loss) memcpy(loss, n->hret + n->ret_loss, sizeof(double));
+    return net_status_value(n);
 }
 
 sim_status sim_net_train_step(sim_net_t *n, const float *x_dev, const float *target_dev, float lr, double *loss) {
@@ -1003,7 +1051,7 @@ sim_status sim_net_train_step(sim_net_t *n, const float *x_dev, const float *tar
     if (n->err != SIM_OK) return n->err;
     features_kernel<<<sim_blocks(n->d.N), SIM_THREADS, 0, n->stream>>>(n->d, x_dev, (uint16_t *)n->act[0], nullptr);
     NET_LAUNCHED(n);
-    if (net_forward(n) != SIM_OK || net_backward(n, target_dev) != SIM_OK) return n->err;
+    if (net_forward(n, n->out) != SIM_OK || net_backward(n, target_dev) != SIM_OK) return n->err;
     n->adam_t++;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)n->adam_t), c2 = 1.f - std::pow(b2, (float)n->adam_t);
@@ -1042,10 +1090,10 @@ sim_status sim_net_time_conv(sim_net_t *n, int32_t which, int32_t reps, double *
                 nullptr, n->dstat, -1);
         } else if (which == 1) {
             wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[0], n->d,
-                                                                           wg_bricks(n->d), n->wpart, n->dstat);
+                                                                           wg_run(n->d), COUT[l], n->wpart, n->dstat);
             n->launches++;
-            wgrad_fold_kernel<<<sim_blocks(27 * 256), SIM_THREADS, 0, n->stream>>>(n->wg_ctas, CIN[l], COUT[l], n->wpart,
-                                                                                    n->grad + n->off_w[l]);
+            wgrad_fold_kernel<<<sim_blocks(27 * CIN[l] * COUT[l] + COUT[l], 32), 256, 0, n->stream>>>(
+                n->wg_ctas, CIN[l], COUT[l], n->wpart, n->grad + n->off_w[l]);
         } else {
             conv_tc_kernel<2><<<tc_grid(n->d), TC_THREADS, TC_SMEM, n->stream>>>(
                 n->map_g[0], n->d, tc_bricks(n->d), n->wb[l], nullptr, n->act[l], n->g1, nullptr, nullptr, n->dstat, -1);
@@ -1077,9 +1125,7 @@ sim_status net_infer(sim_net_t *n, const float *x_dev, float *y_dev, cudaStream_
     n->stream = st;
     features_kernel<<<sim_blocks(n->d.N), SIM_THREADS, 0, st>>>(n->d, x_dev, (uint16_t *)n->act[0], done);
     n->launches++;
-    sim_status r = net_forward(n, done);
-    if (r == SIM_OK && cudaMemcpyAsync(y_dev, n->out, sizeof(float) * n->d.N, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        r = SIM_ECUDA;
+    sim_status r = net_forward(n, y_dev, done);
     n->stream = keep;
     return r;
 }
@@ -1087,9 +1133,10 @@ int64_t net_launches(sim_net_t *n) { return n ? n->launches : 0; }
 int net_status_word(sim_net_t *n, cudaStream_t st) {
     int v = 0;
     if (!n) return 0;
-    if (cudaMemcpyAsync(&v, n->dstat, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(n->hret + n->ret_stat, n->dstat, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return -1;
+    memcpy(&v, n->hret + n->ret_stat, sizeof(int));
     return v;
 }
 int net_cells(sim_net_t *n) { return n ? n->d.N : 0; }
