@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -1411,14 +1412,18 @@ __global__ void amg_smooth_kernel(Mat<T> A, const T *__restrict__ f, const T *__
 
 // next stage-P cycle: f0 = rp - A_p ep; e0 = f0 / l1
 template <typename T>
+__device__ __forceinline__ void cycle_next_row(const Mat<T> &A, const T *__restrict__ rp, const T *__restrict__ ep,
+                                               const T *__restrict__ dinv, T *__restrict__ f0, T *__restrict__ e0, int i) {
+    const T f = rp[i] - row_dot(A, i, ep);
+    f0[i] = f;
+    e0[i] = f * dinv[i];
+}
+template <typename T>
 __global__ void cycle_next_kernel(Mat<T> A, const T *__restrict__ rp, const T *__restrict__ ep, const T *__restrict__ dinv,
                                   T *__restrict__ f0, T *__restrict__ e0, const int *done) {
     if (skip(done)) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.n) return;
-    const T f = rp[i] - row_dot(A, i, ep);
-    f0[i] = f;
-    e0[i] = f * dinv[i];
+    if (i < A.n) cycle_next_row<T>(A, rp, ep, dinv, f0, e0, i);
 }
 
 // y = x (mode 0) or y += x (mode 1)
@@ -1534,7 +1539,7 @@ __device__ __forceinline__ void coarse_cycle_body(const CoarseCycle<T> &cc, int 
     }
     for (int l = 0; l < last; l++) {
         const CoarseLevel<T> &L = cc.lv[l], &C = cc.lv[l + 1];
-        const int lanes = ell_lanes(L.n);
+        const int lanes = L.st ? 1 : ell_lanes(L.n);
         sweep_rows(L.n, lanes, rank, nb, [&](int i, bool ok, int sub) {
             const T t = coarse_dot<T>(cc, L, i, ok, lanes, sub, ok ? L.e[i] : (T)0, [&](int j) { return L.e[j]; });
             if (ok && sub == 0) L.e2[i] = L.f[i] - t;
@@ -1575,7 +1580,7 @@ __device__ __forceinline__ void coarse_cycle_body(const CoarseCycle<T> &cc, int 
     for (int l = last - 1; l >= 0; l--) {
         const CoarseLevel<T> &L = cc.lv[l], &C = cc.lv[l + 1];
         const T *ec = (l + 1 == last) ? C.e : C.e2;
-        const int lanes = ell_lanes(L.n);
+        const int lanes = L.st ? 1 : ell_lanes(L.n);
         sweep_rows(L.n, lanes, rank, nb, [&](int i, bool ok, int sub) {
             auto e = [&](int j) { return L.e[j] + ec[L.agg[j]]; };
             const T ei = ok ? e(i) : (T)0;
@@ -1665,15 +1670,11 @@ __global__ void stage2_a_kernel(GridDesc g, const double *__restrict__ r, const 
 // CPR-FPF, after the first stage F (x0): rh = L r - Ahat x0 over the full 7-point
 // block stencil; f0 = rh_p, e0 = f0 / l1 start stage P
 template <int B, typename T>
-__global__ void fpf_resid_kernel(GridDesc g, const double *__restrict__ r, const T *__restrict__ wT,
-                                 const T *__restrict__ lscT, const T *__restrict__ ahat, const T *__restrict__ x0,
-                                 const T *__restrict__ dinv0, T *__restrict__ rh, T *__restrict__ f0, T *__restrict__ e0,
-                                 const L2Prefetch pf, const int *done) {
-    if (skip(done)) return;
-    issue_prefetch(pf);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void fpf_resid_row(const GridDesc &g, const double *__restrict__ r, const T *__restrict__ wT,
+                                              const T *__restrict__ lscT, const T *__restrict__ ahat,
+                                              const T *__restrict__ x0, const T *__restrict__ dinv0, T *__restrict__ rh,
+                                              T *__restrict__ f0, T *__restrict__ e0, int i) {
     const long N = g.N;
-    if (i >= N) return;
     T v[B], u[B];
 #pragma unroll
     for (int c = 0; c < B; c++) u[c] = (T)r[(long)c * N + i];
@@ -1709,6 +1710,17 @@ __global__ void fpf_resid_kernel(GridDesc g, const double *__restrict__ r, const
     for (int c = 0; c < B; c++) rh[(long)c * N + i] = v[c];
     f0[i] = v[0];
     e0[i] = v[0] * dinv0[i];
+}
+
+template <int B, typename T>
+__global__ void fpf_resid_kernel(GridDesc g, const double *__restrict__ r, const T *__restrict__ wT,
+                                 const T *__restrict__ lscT, const T *__restrict__ ahat, const T *__restrict__ x0,
+                                 const T *__restrict__ dinv0, T *__restrict__ rh, T *__restrict__ f0, T *__restrict__ e0,
+                                 const L2Prefetch pf, const int *done) {
+    if (skip(done)) return;
+    issue_prefetch(pf);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < g.N) fpf_resid_row<B, T>(g, r, wT, lscT, ahat, x0, dinv0, rh, f0, e0, i);
 }
 
 // stage-F output of component r: x (+ e_p on the pressure row) (+ addv, the first
@@ -1812,6 +1824,92 @@ __global__ void stage2_c_kernel(GridDesc g, const T *__restrict__ ahat, const T 
                      : (blockIdx.x * blockDim.x + threadIdx.x < (unsigned)g.N ? (int)(blockIdx.x * blockDim.x + threadIdx.x) : -1);
     if (i < 0) return;
     stage2_c_row<B, T, TZ>(g, ahat, dinv, z, ep, addv, out, rb, i);
+}
+
+// ---- the whole CPR application of a small grid in one launch -----------------
+// Up to kSmallCells cells an application is 10 to 25 dependent launches of 2.5 to 5 us
+// each, whose work is a fraction of that; here they are sweeps of one 16-CTA cluster with a
+// cluster barrier (about 1 us) between them, calling the same row functions in the
+// same order, level 0 of the V-cycle among them, so the result is that of the
+// separate launches bit for bit.  2,000 two-phase cells: an application 72 -> 48 us, an
+// FGMRES iteration (its launches replayed from a graph) 86 -> 77 us.  The latency of
+// 16 SMs sets the bound: an iteration at 4,000 cells goes from 82 to 78 us, at 7,840
+// from 88 to 92.
+constexpr int kSmallCells = 5120, kSmallThreads = 512;
+
+template <typename T>
+struct SmallApply {
+    CoarseCycle<T> cc;                 // every level
+    const T *wT, *lscT, *ahat, *dinv;
+    T *r2, *zr, *x0, *rhT, *rpT, *epacc;
+    int full, rb, fpf, cycles;
+};
+
+// out = M r by CTA `rank` of the nb CTAs of one cluster
+template <int B, typename T, typename TZ>
+__device__ __forceinline__ void small_apply_body(const SmallApply<T> &S, const double *__restrict__ r, TZ *__restrict__ out,
+                                                 int rank, int nb) {
+    const GridDesc &g = S.cc.g;
+    const CoarseLevel<T> &L0 = S.cc.lv[0];
+    const int N = g.N, slots = g.H;
+    const bool one = S.cc.nlev == 1;   // a single level is solved by its dense inverse
+    auto cells = [&](int n, auto f) {
+        const int per = (n + nb - 1) / nb, hi = min(n, (rank + 1) * per);
+        for (int i = rank * per + (int)threadIdx.x; i < hi; i += kSmallThreads) f(i);
+    };
+    // one stage F (three sweeps) into o
+    auto stage_f = [&](const double *ri, const T *rh, const T *ep, const T *addv, auto *o) {
+        using TO = std::remove_pointer_t<decltype(o)>;
+        cells(N, [&](int i) { stage2_a_row<B, T>(g, ri, S.wT, S.lscT, rh, S.ahat, S.dinv, ep, S.r2, S.zr, S.rb, i); });
+        cluster_barrier();
+        if (S.rb) {
+            cells(slots, [&](int t) {
+                const int i = colour_cell(g, t, 1);
+                if (i >= 0) stage2_b_row<B, T, TO>(g, S.ahat, S.dinv, S.r2, S.zr, ep, addv, o, i);
+            });
+            cluster_barrier();
+            cells(slots, [&](int t) {
+                const int i = colour_cell(g, t, 0);
+                if (i >= 0) stage2_c_row<B, T, TO>(g, S.ahat, S.dinv, S.zr, ep, addv, o, 1, i);
+            });
+        } else {
+            cells(N, [&](int i) { stage2_c_row<B, T, TO>(g, S.ahat, S.dinv, S.zr, ep, addv, o, 0, i); });
+        }
+    };
+    if (S.fpf) {
+        stage_f(r, (const T *)nullptr, (const T *)nullptr, (const T *)nullptr, S.x0);
+        cluster_barrier();
+        cells(N, [&](int i) { fpf_resid_row<B, T>(g, r, S.wT, S.lscT, S.ahat, S.x0, L0.dinv, S.rhT, L0.f, L0.e, i); });
+    } else {
+        cells(N, [&](int i) { restrict_p_row<B, T>(N, r, S.wT, S.full, L0.dinv, L0.f, L0.e, i); });
+    }
+    cluster_barrier();
+    coarse_cycle_body<T>(S.cc, rank, nb);
+    const T *ep = one ? L0.e : L0.e2;
+    if (S.cycles > 1 && !one) {
+        cluster_barrier();
+        cells(N, [&](int i) { S.rpT[i] = L0.f[i]; S.epacc[i] = L0.e2[i]; });
+        Mat<T> A;
+        A.st = true; A.selfpad = true; A.diff = L0.diff != 0; A.g = g; A.val = L0.val; A.col = nullptr; A.n = N; A.width = 7;
+        for (int c = 1; c < S.cycles; c++) {
+            cluster_barrier();
+            cells(N, [&](int i) { cycle_next_row<T>(A, S.rpT, S.epacc, L0.dinv, L0.f, L0.e, i); });
+            cluster_barrier();
+            coarse_cycle_body<T>(S.cc, rank, nb);
+            cluster_barrier();
+            cells(N, [&](int i) { S.epacc[i] = S.epacc[i] + L0.e2[i]; });
+        }
+        ep = S.epacc;
+    }
+    cluster_barrier();
+    stage_f(S.fpf ? nullptr : r, S.rhT, ep, S.fpf ? S.x0 : (const T *)nullptr, out);
+}
+
+template <int B, typename T, typename TZ>
+__global__ void __launch_bounds__(kSmallThreads, 1) small_apply_kernel(const __grid_constant__ SmallApply<T> S,
+                                                                      const double *r, TZ *out, const int *done) {
+    if (skip(done)) return;            // uniform over the cluster
+    small_apply_body<B, T, TZ>(S, r, out, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // no preconditioner / plain block-Jacobi on J (no decoupling)
@@ -2401,10 +2499,10 @@ static L2Prefetch coarse_prefetch(const sim_t *s) {
     return pf;
 }
 
-// a launch of `clusters` clusters of 16 CTAs of kCoarseThreads, or of 8 where an
+// a launch of `clusters` clusters of 16 CTAs, or of 8 where an
 // occupancy query finds no room for 16 (a non-portable size); the query launches nothing
 template <typename... KArgs>
-static int coarse_ctas(void (*kernel)(KArgs...)) {
+static int coarse_ctas(void (*kernel)(KArgs...), int threads) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         (void)cudaGetLastError();
         return 8;
@@ -2413,7 +2511,7 @@ static int coarse_ctas(void (*kernel)(KArgs...)) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 16; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(16); cfg.blockDim = dim3(kCoarseThreads);
+    cfg.gridDim = dim3(16); cfg.blockDim = dim3(threads);
     cfg.attrs = at; cfg.numAttrs = 1;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
@@ -2422,16 +2520,16 @@ static int coarse_ctas(void (*kernel)(KArgs...)) {
     }
     return n > 0 ? 16 : 8;
 }
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_clusters(void (*kernel)(KArgs...), int clusters, cudaStream_t st, Args &&...args) {
-    static const int ctas = coarse_ctas(kernel);      // one per kernel (per instantiation of its type)
+template <auto Kernel, typename... Args>
+static cudaError_t launch_clusters(int clusters, int threads, cudaStream_t st, Args... args) {
+    static const int ctas = coarse_ctas(Kernel, threads);      // per kernel: its attributes are its own
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(clusters * ctas); cfg.blockDim = dim3(kCoarseThreads); cfg.stream = st;
+    cfg.gridDim = dim3(clusters * ctas); cfg.blockDim = dim3(threads); cfg.stream = st;
     cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return cudaLaunchKernelEx(&cfg, Kernel, args...);
 }
 
 template <typename T>
@@ -2442,6 +2540,23 @@ static CoarseLevel<T> coarse_level(const AmgLevel &L, int l) {
     d.agg = L.agg; d.moff = L.moff; d.mem = L.mem;
     d.f = (T *)L.f; d.e = (T *)L.e; d.e2 = (T *)L.e2;
     return d;
+}
+
+// the one-launch application of a small grid
+static bool small_grid(const sim_t *s) {
+    return s->N <= kSmallCells && s->opt.fused_coarse && (int)s->lev.size() <= kCoarseMaxLevels;
+}
+template <typename T>
+static SmallApply<T> small_apply(const sim_t *s) {
+    SmallApply<T> S;
+    S.cc.nlev = (int)s->lev.size(); S.cc.g = s->gd; S.cc.inv = (const double *)s->lev.back().coarse_inv;
+    for (size_t l = 0; l < s->lev.size(); l++) S.cc.lv[l] = coarse_level<T>(s->lev[l], (int)l);
+    S.full = s->opt.decouple == SIM_DECOUPLE_ABF;
+    S.wT = (const T *)s->qiwT; S.lscT = S.full ? (const T *)s->lscT : nullptr; S.ahat = (const T *)s->ahat;
+    S.dinv = sizeof(T) == sizeof(double) ? (const T *)s->dinv_d : (const T *)s->dinv;
+    S.r2 = (T *)s->r2; S.zr = (T *)s->zr; S.x0 = (T *)s->x0; S.rhT = (T *)s->rhT; S.rpT = (T *)s->rpT; S.epacc = (T *)s->epacc;
+    S.rb = s->opt.stage2 == SIM_STAGE2_ILU0_RB; S.fpf = s->opt.cpr_stages == 3; S.cycles = s->opt.amg_cycles;
+    return S;
 }
 
 template <typename T>
@@ -2455,7 +2570,7 @@ static sim_status coarse_cycle(sim_t *s, int l0, const int *done) {
         CoarseLevel<T> &d = cc.lv[l - l0];
         d = coarse_level<T>(L, l);
     }
-    if (!sim_cuda_ok(s, launch_clusters(coarse_cycle_kernel<T>, 1, s->stream, cc, done), "coarse cycle")) return s->err;
+    if (!sim_cuda_ok(s, launch_clusters<coarse_cycle_kernel<T>>(1, kCoarseThreads, s->stream, cc, done), "coarse cycle")) return s->err;
     SIM_LAUNCHED(s);
     return SIM_OK;
 }
@@ -2514,6 +2629,13 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
     const int full = s->opt.decouple == SIM_DECOUPLE_ABF;
     const T *lscT = full ? (const T *)s->lscT : nullptr;
     const bool fpf = s->opt.cpr_stages == 3;
+    if (small_grid(s) && !s->learned_active) {
+        if (!sim_cuda_ok(s, launch_clusters<small_apply_kernel<B, T, TZ>>(1, kSmallThreads, s->stream, small_apply<T>(s), r, z, done),
+                         "CPR application"))
+            return s->err;
+        SIM_LAUNCHED(s);
+        return SIM_OK;
+    }
     if (fpf) {
         // CPR-FPF: stage F on L r first (x0), then stage P on the residual it leaves
         stage2_a_kernel<B, T><<<sim_blocks(N, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, r, (const T *)s->qiwT, lscT, nullptr,
@@ -2727,6 +2849,23 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) b_coarse_cycle_kernel(const
     coarse_cycle_body<T>(*m.cc, (int)(blockIdx.x % nb), nb);
 }
 
+// whole applications of small members: cluster c runs tab[c]
+template <typename T>
+struct SmallMember {
+    SmallApply<T> S;
+    const double *V;            // input of application j: V + j n (FP64)
+    T *Z;                       // output: Z + j n
+    long n;
+    const int *done;
+};
+template <int B, typename T>
+__global__ void __launch_bounds__(kSmallThreads, 1) b_small_apply_kernel(const SmallMember<T> *tab, int j) {
+    const int nb = (int)cg::this_cluster().num_blocks();
+    const SmallMember<T> &m = tab[blockIdx.x / nb];
+    if (skip(m.done)) return;          // uniform over the cluster (one member)
+    small_apply_body<B, T, T>(m.S, m.V + (size_t)j * m.n, m.Z + (size_t)j * m.n, (int)(blockIdx.x % nb), nb);
+}
+
 // stage F on the residual of stage P: sweep 0 (all cells), 1 (black), 2 (red,
 // or all cells for block Jacobi)
 template <int B, typename T>
@@ -2756,7 +2895,8 @@ struct CprBatch {
     void *dcc = nullptr;   size_t cc_cap = 0;     // CoarseCycle<T>[ncl]
     int2 *dwork = nullptr; size_t work_cap = 0;
     int *dcl = nullptr;    size_t cl_cap = 0;     // members with fused coarse levels
-    int ncl = 0;
+    void *dsmall = nullptr; size_t small_cap = 0; // SmallMember<T>[nsmall]
+    int ncl = 0, nsmall = 0;
     struct List { long off = 0; int count = 0; };
     List cell256, cell64, stage1, stage2, cs;
     std::vector<List> down_r, down_c, up, up_s;
@@ -2794,11 +2934,18 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
     std::vector<CoarseCycle<T>> hcc;
     std::vector<int> hcl;
     std::vector<int2> work;
+    std::vector<SmallMember<T>> hsm;
+    // up to eight small members take an application in one launch, a cluster each (as
+    // many as are resident at once); more of them fill the GPU as rows of the others do
+    int nsmall = 0;
+    for (int k = 0; k < nm; k++) nsmall += small_grid(ms[k]) ? 1 : 0;
+    std::vector<char> small(nm, 0);
+    for (int k = 0; k < nm; k++) small[k] = nsmall <= 8 && small_grid(ms[k]);
     cb->down_r.clear(); cb->down_c.clear(); cb->up.clear(); cb->up_s.clear();
     auto add_list = [&](CprBatch::List &L, auto blocks_of) {
         L.off = (long)work.size();
         for (int k = 0; k < nm; k++) {
-            const int nb = blocks_of(k);
+            const int nb = small[k] ? 0 : blocks_of(k);
             for (int q = 0; q < nb; q++) work.push_back(make_int2(k, q));
         }
         L.count = (int)((long)work.size() - L.off);
@@ -2829,6 +2976,10 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
             d.A = level_matT<T>(s, L, l);
             d.dinv = (const T *)L.dinvT; d.agg = L.agg; d.moff = L.moff; d.mem = L.mem;
             d.f = (T *)L.f; d.e = (T *)L.e; d.e2 = (T *)L.e2; d.n = L.n;
+        }
+        if (small[k]) {
+            hsm.push_back(SmallMember<T>{small_apply<T>(s), s->V, (T *)s->Z, m.n, m.done});
+            continue;
         }
         if (m.lf < nl) {
             CoarseCycle<T> cc;
@@ -2875,6 +3026,11 @@ static cudaError_t batch_build_t(CprBatch *cb, sim_t *const *ms, int nm, cudaStr
         if ((e = cudaMemcpyAsync(cb->dcl, hcl.data(), sizeof(int) * hcl.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     }
     cb->ncl = (int)hcl.size();
+    if (!hsm.empty()) {
+        if ((e = grow(&cb->dsmall, &cb->small_cap, sizeof(SmallMember<T>) * hsm.size())) != cudaSuccess) return e;
+        if ((e = cudaMemcpyAsync(cb->dsmall, hsm.data(), sizeof(SmallMember<T>) * hsm.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
+    }
+    cb->nsmall = (int)hsm.size();
     if ((e = cudaMemcpyAsync(cb->dmem, hm.data(), sizeof(CMember<T>) * nm, cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     if (!work.empty() && (e = cudaMemcpyAsync(cb->dwork, work.data(), sizeof(int2) * work.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     // the host tables must outlive the asynchronous copies
@@ -2891,6 +3047,7 @@ void cpr_batch_free(CprBatch *cb) {
     if (cb->dcc) cudaFree(cb->dcc);
     if (cb->dwork) cudaFree(cb->dwork);
     if (cb->dcl) cudaFree(cb->dcl);
+    if (cb->dsmall) cudaFree(cb->dsmall);
     delete cb;
 }
 
@@ -2906,13 +3063,18 @@ static int batch_apply_t(const CprBatch *cb, cudaStream_t st, int j) {
     auto go = [&](const CprBatch::List &L, int threads, auto launch) {
         if (L.count > 0) { launch(L.count, threads, W + L.off); launches++; }
     };
+    if (cb->nsmall > 0) {
+        if (launch_clusters<b_small_apply_kernel<B, T>>(cb->nsmall, kSmallThreads, st, (const SmallMember<T> *)cb->dsmall, j) != cudaSuccess)
+            return -1;
+        launches++;
+    }
     go(cb->cell256, SIM_THREADS, [&](int n, int t, const int2 *w) { b_restrict_p_kernel<B, T><<<n, t, 0, st>>>(M, w, j); });
     for (size_t l = 0; l < cb->down_r.size(); l++) {
         go(cb->down_r[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_down_kernel<T><<<n, t, 0, st>>>(M, w, (int)l, 0); });
         go(cb->down_c[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_down_kernel<T><<<n, t, 0, st>>>(M, w, (int)l, 1); });
     }
     if (cb->ncl > 0) {
-        if (launch_clusters(b_coarse_cycle_kernel<T>, cb->ncl, st, M, (const int *)cb->dcl) != cudaSuccess) return -1;
+        if (launch_clusters<b_coarse_cycle_kernel<T>>(cb->ncl, kCoarseThreads, st, M, (const int *)cb->dcl) != cudaSuccess) return -1;
         launches++;
     }
     go(cb->cs, SIM_THREADS, [&](int n, int t, const int2 *w) { b_coarse_solve_kernel<T><<<n, t, 0, st>>>(M, w); });
