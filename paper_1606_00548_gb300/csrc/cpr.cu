@@ -36,7 +36,11 @@ namespace {
 
 constexpr int MAXE = SIM_MAX_ELL;
 
-__device__ __forceinline__ bool skip(const int *done) { return done != nullptr && *(volatile const int *)done; }
+// enter (see sim_launch) and test the flag
+__device__ __forceinline__ bool skip(const int *done) {
+    sim_enter();
+    return done != nullptr && *(volatile const int *)done;
+}
 
 struct Cell { int i, ix, iy, iz; };
 __device__ __forceinline__ Cell cell_of(const GridDesc &g, int i) {
@@ -2535,11 +2539,13 @@ template <auto Kernel, typename... Args>
 static cudaError_t launch_clusters(int clusters, int threads, cudaStream_t st, Args... args) {
     static const int ctas = coarse_ctas(Kernel, threads);      // per kernel: its attributes are its own
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // as sim_launch
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(clusters * ctas); cfg.blockDim = dim3(threads); cfg.stream = st;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    cfg.attrs = at; cfg.numAttrs = sim_overlaps(st) ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, Kernel, args...);
 }
 
@@ -2595,10 +2601,10 @@ static sim_status vcycle(sim_t *s, const int *done, T *acc = nullptr) {
     for (int l = 0; l + 1 < nl && l < lf; l++) {
         AmgLevel &L = s->lev[l], &C = s->lev[l + 1];
         const bool coarsest = (l + 1 == nl - 1);
-        amg_resid_kernel<T><<<level_blocks(L.n, l, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
+        sim_launch(amg_resid_kernel<T>, level_blocks(L.n, l, s->tune_amg), s->tune_amg, s->stream, level_matT<T>(s, L, l), (const T *)L.f,
                                                                         (const T *)L.e, (T *)L.e2, done);
         SIM_LAUNCHED(s);
-        amg_restrict_kernel<T><<<sim_blocks(C.n, s->tune_amg), s->tune_amg, 0, s->stream>>>((const T *)L.e2, L.moff, L.mem, C.n, (T *)C.f,
+        sim_launch(amg_restrict_kernel<T>, sim_blocks(C.n, s->tune_amg), s->tune_amg, s->stream, (const T *)L.e2, L.moff, L.mem, C.n, (T *)C.f,
                                                                            coarsest ? nullptr : (T *)C.e,
                                                                            (const T *)C.dinvT, done);
         SIM_LAUNCHED(s);
@@ -2607,7 +2613,7 @@ static sim_status vcycle(sim_t *s, const int *done, T *acc = nullptr) {
         if (coarse_cycle<T>(s, lf, done) != SIM_OK) return s->err;
     } else {
         AmgLevel &Cn = s->lev[nl - 1];
-        coarse_solve_kernel<T><<<sim_blocks((long)Cn.n * 32), SIM_THREADS, 0, s->stream>>>(Cn.n, (const double *)Cn.coarse_inv,
+        sim_launch(coarse_solve_kernel<T>, sim_blocks((long)Cn.n * 32), SIM_THREADS, s->stream, Cn.n, (const double *)Cn.coarse_inv,
                                                                                         (const T *)Cn.f, (T *)Cn.e, done);
         SIM_LAUNCHED(s);
     }
@@ -2615,16 +2621,16 @@ static sim_status vcycle(sim_t *s, const int *done, T *acc = nullptr) {
     for (int l = (lf < nl ? lf : nl - 1) - 1; l >= 0; l--) {
         AmgLevel &L = s->lev[l], &C = s->lev[l + 1];
         const T *ec = (l + 1 == nl - 1) ? (const T *)C.e : (const T *)C.e2;
-        amg_prolong_kernel<T><<<sim_blocks(L.n, s->tune_amg), s->tune_amg, 0, s->stream>>>(L.n, L.agg, ec, (T *)L.e, done);
+        sim_launch(amg_prolong_kernel<T>, sim_blocks(L.n, s->tune_amg), s->tune_amg, s->stream, L.n, L.agg, ec, (T *)L.e, done);
         SIM_LAUNCHED(s);
         const bool add = l == 0 && acc;
-        amg_smooth_kernel<T><<<level_blocks(L.n, l, s->tune_amg), s->tune_amg, 0, s->stream>>>(level_matT<T>(s, L, l), (const T *)L.f,
+        sim_launch(amg_smooth_kernel<T>, level_blocks(L.n, l, s->tune_amg), s->tune_amg, s->stream, level_matT<T>(s, L, l), (const T *)L.f,
                                                                          (const T *)L.e, (const T *)L.dinvT,
                                                                          add ? acc : (T *)L.e2, done, add);
         SIM_LAUNCHED(s);
     }
     if (acc && lf == 0) {
-        copy_add_kernel<T><<<sim_blocks(s->N), SIM_THREADS, 0, s->stream>>>(s->N, (const T *)s->lev[0].e2, acc, 1, done);
+        sim_launch(copy_add_kernel<T>, sim_blocks(s->N), SIM_THREADS, s->stream, s->N, (const T *)s->lev[0].e2, acc, 1, done);
         SIM_LAUNCHED(s);
     }
     return SIM_OK;
@@ -2635,7 +2641,7 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
     const int N = s->N;
     const int nb = sim_blocks(N);
     if (s->opt.precond != SIM_PRECOND_CPR) {
-        simple_prec_kernel<B, TZ><<<nb, SIM_THREADS, 0, s->stream>>>(s->gd, r, s->dinv_d, z,
+        sim_launch(simple_prec_kernel<B, TZ>, nb, SIM_THREADS, s->stream, s->gd, r, s->dinv_d, z,
                                                                    s->opt.precond == SIM_PRECOND_BJACOBI, done);
         SIM_LAUNCHED(s);
         return SIM_OK;
@@ -2655,30 +2661,30 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
     }
     if (fpf) {
         // CPR-FPF: stage F on L r first (x0), then stage P on the residual it leaves
-        stage2_a_kernel<B, T><<<sim_blocks(N, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, r, (const T *)s->qiwT, lscT, nullptr,
+        sim_launch(stage2_a_kernel<B, T>, sim_blocks(N, s->tune_stage), s->tune_stage, s->stream, s->gd, r, (const T *)s->qiwT, lscT, nullptr,
                                                                 (const T *)s->ahat, dinv, nullptr, (T *)s->r2,
                                                                 (T *)s->zr, rb, done);
         SIM_LAUNCHED(s);
         if (rb) {
-            stage2_b_kernel<B, T, T><<<colour_blocks(s, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, (const T *)s->ahat, dinv, (const T *)s->r2,
+            sim_launch(stage2_b_kernel<B, T, T>, colour_blocks(s, s->tune_stage), s->tune_stage, s->stream, s->gd, (const T *)s->ahat, dinv, (const T *)s->r2,
                                                                        (T *)s->zr, nullptr, nullptr, (T *)s->x0, done);
             SIM_LAUNCHED(s);
         }
-        stage2_c_kernel<B, T, T><<<rb ? colour_blocks(s, s->tune_stage) : sim_blocks(N, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, (const T *)s->ahat, dinv, (const T *)s->zr,
+        sim_launch(stage2_c_kernel<B, T, T>, rb ? colour_blocks(s, s->tune_stage) : sim_blocks(N, s->tune_stage), s->tune_stage, s->stream, s->gd, (const T *)s->ahat, dinv, (const T *)s->zr,
                                                                    nullptr, nullptr, (T *)s->x0, rb, done);
         SIM_LAUNCHED(s);
-        fpf_resid_kernel<B, T><<<nb, SIM_THREADS, 0, s->stream>>>(s->gd, r, (const T *)s->qiwT, lscT, (const T *)s->ahat,
+        sim_launch(fpf_resid_kernel<B, T>, nb, SIM_THREADS, s->stream, s->gd, r, (const T *)s->qiwT, lscT, (const T *)s->ahat,
                                                                  (const T *)s->x0, (const T *)L0.dinvT, (T *)s->rhT,
                                                                  (T *)L0.f, (T *)L0.e, coarse_prefetch<T>(s), done);
         SIM_LAUNCHED(s);
     } else {
-        restrict_p_kernel<B, T><<<nb, SIM_THREADS, 0, s->stream>>>(N, r, (const T *)s->qiwT, full, (const T *)L0.dinvT,
+        sim_launch(restrict_p_kernel<B, T>, nb, SIM_THREADS, s->stream, N, r, (const T *)s->qiwT, full, (const T *)L0.dinvT,
                                                                   (T *)L0.f, (T *)L0.e, coarse_prefetch<T>(s), done);
         SIM_LAUNCHED(s);
     }
     const T *ep;
     if (s->lev.size() == 1) {
-        coarse_solve_kernel<T><<<sim_blocks((long)L0.n * 32), SIM_THREADS, 0, s->stream>>>(L0.n, (const double *)L0.coarse_inv,
+        sim_launch(coarse_solve_kernel<T>, sim_blocks((long)L0.n * 32), SIM_THREADS, s->stream, L0.n, (const double *)L0.coarse_inv,
                                                                                         (const T *)L0.f, (T *)L0.e2, done);
         SIM_LAUNCHED(s);
     } else if (vcycle<T>(s, done) != SIM_OK) {
@@ -2690,7 +2696,7 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
         const bool keep = s->opt.amg_cycles > 2 || (s->learned_active && s->net);   // someone reads rpT
         for (int c = 1; c < s->opt.amg_cycles; c++) {
             const bool first = c == 1;
-            cycle_next_kernel<T><<<sim_blocks(N, 128), 128, 0, s->stream>>>(
+            sim_launch(cycle_next_kernel<T>, sim_blocks(N, 128), 128, s->stream,
                 level_matT<T>(s, L0, 0), (const T *)(first ? L0.f : s->rpT), (const T *)(first ? L0.e2 : s->epacc),
                 (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, first && keep ? (T *)s->rpT : nullptr,
                 first ? (T *)s->epacc : nullptr, done);
@@ -2702,7 +2708,7 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
     if (s->learned_active && s->net) {
         // extra stage: the network's correction of the pressure residual left by stage P
         const T *rp = (s->opt.amg_cycles > 1 && s->lev.size() > 1) ? (const T *)s->rpT : (const T *)L0.f;
-        amg_resid_kernel<T><<<sim_blocks(N, 128), 128, 0, s->stream>>>(level_matT<T>(s, L0, 0), rp, ep, (T *)s->lres, done);
+        sim_launch(amg_resid_kernel<T>, sim_blocks(N, 128), 128, s->stream, level_matT<T>(s, L0, 0), rp, ep, (T *)s->lres, done);
         SIM_LAUNCHED(s);
         rms_kernel<T><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(N, (const T *)s->lres, s->red, s->ticket, s->lrms, done);
         SIM_LAUNCHED(s);
@@ -2723,16 +2729,16 @@ static sim_status apply_btz(sim_t *s, const double *r, TZ *z, const int *done) {
         ep = (const T *)s->lep;
     }
     const T *addv = fpf ? (const T *)s->x0 : nullptr;
-    stage2_a_kernel<B, T><<<sim_blocks(N, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, fpf ? nullptr : r, (const T *)s->qiwT, lscT,
+    sim_launch(stage2_a_kernel<B, T>, sim_blocks(N, s->tune_stage), s->tune_stage, s->stream, s->gd, fpf ? nullptr : r, (const T *)s->qiwT, lscT,
                                                             (const T *)s->rhT, (const T *)s->ahat, dinv, ep, (T *)s->r2,
                                                             (T *)s->zr, rb, done);
     SIM_LAUNCHED(s);
     if (rb) {
-        stage2_b_kernel<B, T, TZ><<<colour_blocks(s, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, (const T *)s->ahat, dinv, (const T *)s->r2,
+        sim_launch(stage2_b_kernel<B, T, TZ>, colour_blocks(s, s->tune_stage), s->tune_stage, s->stream, s->gd, (const T *)s->ahat, dinv, (const T *)s->r2,
                                                                     (T *)s->zr, ep, addv, z, done);
         SIM_LAUNCHED(s);
     }
-    stage2_c_kernel<B, T, TZ><<<rb ? colour_blocks(s, s->tune_stage) : sim_blocks(N, s->tune_stage), s->tune_stage, 0, s->stream>>>(s->gd, (const T *)s->ahat, dinv, (const T *)s->zr, ep, addv,
+    sim_launch(stage2_c_kernel<B, T, TZ>, rb ? colour_blocks(s, s->tune_stage) : sim_blocks(N, s->tune_stage), s->tune_stage, s->stream, s->gd, (const T *)s->ahat, dinv, (const T *)s->zr, ep, addv,
                                                                 z, rb, done);
     SIM_LAUNCHED(s);
     return SIM_OK;
@@ -3083,23 +3089,23 @@ static int batch_apply_t(const CprBatch *cb, cudaStream_t st, int j) {
             return -1;
         launches++;
     }
-    go(cb->cell256, SIM_THREADS, [&](int n, int t, const int2 *w) { b_restrict_p_kernel<B, T><<<n, t, 0, st>>>(M, w, j); });
+    go(cb->cell256, SIM_THREADS, [&](int n, int t, const int2 *w) { sim_launch(b_restrict_p_kernel<B, T>, n, t, st, M, w, j); });
     for (size_t l = 0; l < cb->down_r.size(); l++) {
-        go(cb->down_r[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_down_kernel<T><<<n, t, 0, st>>>(M, w, (int)l, 0); });
-        go(cb->down_c[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_down_kernel<T><<<n, t, 0, st>>>(M, w, (int)l, 1); });
+        go(cb->down_r[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { sim_launch(b_amg_down_kernel<T>, n, t, st, M, w, (int)l, 0); });
+        go(cb->down_c[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { sim_launch(b_amg_down_kernel<T>, n, t, st, M, w, (int)l, 1); });
     }
     if (cb->ncl > 0) {
         if (launch_clusters<b_coarse_cycle_kernel<T>>(cb->ncl, kCoarseThreads, st, M, (const int *)cb->dcl) != cudaSuccess) return -1;
         launches++;
     }
-    go(cb->cs, SIM_THREADS, [&](int n, int t, const int2 *w) { b_coarse_solve_kernel<T><<<n, t, 0, st>>>(M, w); });
+    go(cb->cs, SIM_THREADS, [&](int n, int t, const int2 *w) { sim_launch(b_coarse_solve_kernel<T>, n, t, st, M, w); });
     for (int l = (int)cb->up.size() - 1; l >= 0; l--) {
-        go(cb->up[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_up_kernel<T><<<n, t, 0, st>>>(M, w, l, 0); });
-        go(cb->up_s[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { b_amg_up_kernel<T><<<n, t, 0, st>>>(M, w, l, 1); });
+        go(cb->up[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { sim_launch(b_amg_up_kernel<T>, n, t, st, M, w, l, 0); });
+        go(cb->up_s[l], kBatchAmgThreads, [&](int n, int t, const int2 *w) { sim_launch(b_amg_up_kernel<T>, n, t, st, M, w, l, 1); });
     }
-    go(cb->cell64, kStageThreads, [&](int n, int t, const int2 *w) { b_stage2_kernel<B, T><<<n, t, 0, st>>>(M, w, j, 0); });
-    go(cb->stage1, kStageThreads, [&](int n, int t, const int2 *w) { b_stage2_kernel<B, T><<<n, t, 0, st>>>(M, w, j, 1); });
-    go(cb->stage2, kStageThreads, [&](int n, int t, const int2 *w) { b_stage2_kernel<B, T><<<n, t, 0, st>>>(M, w, j, 2); });
+    go(cb->cell64, kStageThreads, [&](int n, int t, const int2 *w) { sim_launch(b_stage2_kernel<B, T>, n, t, st, M, w, j, 0); });
+    go(cb->stage1, kStageThreads, [&](int n, int t, const int2 *w) { sim_launch(b_stage2_kernel<B, T>, n, t, st, M, w, j, 1); });
+    go(cb->stage2, kStageThreads, [&](int n, int t, const int2 *w) { sim_launch(b_stage2_kernel<B, T>, n, t, st, M, w, j, 2); });
     return launches;
 }
 
@@ -3137,7 +3143,7 @@ static sim_status learned_pairs_t(sim_t *s, int k, float *x, float *y) {
     const Mat<T> A0 = level_matT<T>(s, L0, 0);
     auto cycle = [&](void) -> sim_status {
         if (s->lev.size() == 1) {
-            coarse_solve_kernel<T><<<sim_blocks((long)L0.n * 32), SIM_THREADS, 0, s->stream>>>(
+            sim_launch(coarse_solve_kernel<T>, sim_blocks((long)L0.n * 32), SIM_THREADS, s->stream,
                 L0.n, (const double *)L0.coarse_inv, (const T *)L0.f, (T *)L0.e2, nullptr);
             SIM_LAUNCHED(s);
             return SIM_OK;
@@ -3146,24 +3152,24 @@ static sim_status learned_pairs_t(sim_t *s, int k, float *x, float *y) {
     };
     for (int j = 0; j < k; j++) {
         const double *v = s->V + (size_t)j * N * s->b;
-        if (s->b == 2) restrict_p_kernel<2, T><<<sim_blocks(N), SIM_THREADS, 0, s->stream>>>(N, v, (const T *)s->qiwT, full, (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, L2Prefetch{}, nullptr);
-        else restrict_p_kernel<3, T><<<sim_blocks(N), SIM_THREADS, 0, s->stream>>>(N, v, (const T *)s->qiwT, full, (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, L2Prefetch{}, nullptr);
+        if (s->b == 2) sim_launch(restrict_p_kernel<2, T>, sim_blocks(N), SIM_THREADS, s->stream, N, v, (const T *)s->qiwT, full, (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, L2Prefetch{}, nullptr);
+        else sim_launch(restrict_p_kernel<3, T>, sim_blocks(N), SIM_THREADS, s->stream, N, v, (const T *)s->qiwT, full, (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, L2Prefetch{}, nullptr);
         SIM_LAUNCHED(s);
         if (cycle() != SIM_OK) return s->err;
         // r' = f - A_p e_p into rpT; the first refinement cycle starts from it
-        amg_resid_kernel<T><<<sim_blocks(N, 128), 128, 0, s->stream>>>(A0, (const T *)L0.f, (const T *)L0.e2, (T *)s->rpT,
+        sim_launch(amg_resid_kernel<T>, sim_blocks(N, 128), 128, s->stream, A0, (const T *)L0.f, (const T *)L0.e2, (T *)s->rpT,
                                                                      nullptr);
         SIM_LAUNCHED(s);
-        copy_add_kernel<T><<<sim_blocks(N), SIM_THREADS, 0, s->stream>>>(N, (const T *)s->rpT, (T *)s->lres, 0, nullptr);
+        sim_launch(copy_add_kernel<T>, sim_blocks(N), SIM_THREADS, s->stream, N, (const T *)s->rpT, (T *)s->lres, 0, nullptr);
         SIM_LAUNCHED(s);
         SIM_CK(s, cudaMemsetAsync(s->epacc, 0, sizeof(T) * (size_t)N, s->stream));
         for (int c = 0; c < kRefine; c++) {
-            cycle_next_kernel<T><<<sim_blocks(N, 128), 128, 0, s->stream>>>(A0, (const T *)s->rpT, (const T *)s->epacc,
+            sim_launch(cycle_next_kernel<T>, sim_blocks(N, 128), 128, s->stream, A0, (const T *)s->rpT, (const T *)s->epacc,
                                                                            (const T *)L0.dinvT, (T *)L0.f, (T *)L0.e, nullptr,
                                                                            nullptr, nullptr);
             SIM_LAUNCHED(s);
             if (cycle() != SIM_OK) return s->err;
-            copy_add_kernel<T><<<sim_blocks(N), SIM_THREADS, 0, s->stream>>>(N, (const T *)L0.e2, (T *)s->epacc, 1, nullptr);
+            sim_launch(copy_add_kernel<T>, sim_blocks(N), SIM_THREADS, s->stream, N, (const T *)L0.e2, (T *)s->epacc, 1, nullptr);
             SIM_LAUNCHED(s);
         }
         rms_kernel<T><<<SIM_RED_BLOCKS, SIM_THREADS, 0, s->stream>>>(N, (const T *)s->lres, s->red, s->ticket, s->lrms, nullptr);

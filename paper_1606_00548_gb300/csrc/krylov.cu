@@ -18,7 +18,11 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-__device__ __forceinline__ bool skip(const int *done) { return done != nullptr && *(volatile const int *)done; }
+// enter (see sim_launch) and test the flag
+__device__ __forceinline__ bool skip(const int *done) {
+    sim_enter();
+    return done != nullptr && *(volatile const int *)done;
+}
 
 template <typename X> __device__ __forceinline__ double ld(const X *p, long i) { return (double)p[i]; }
 
@@ -407,6 +411,7 @@ template <int NV>
 __global__ void __launch_bounds__(kNormThreads, 2) orth_norm_kernel(const double *__restrict__ V, double *__restrict__ w,
                                                                     long n, int j, int m, double *partials,
                                                                     unsigned int *ticket, KrylovCtl *ctl, int selective) {
+    sim_enter();
     if (ctl->done) return;
     orth_norm_body<NV>(V, w, n, j, m, partials, ticket, ctl, selective, grid_blk());
 }
@@ -422,6 +427,7 @@ __device__ __forceinline__ void scale_body(const double *__restrict__ w, double 
 
 __global__ void scale_kernel(const double *__restrict__ w, double *__restrict__ v, long n, const KrylovCtl *ctl,
                              int use_beta) {
+    sim_enter();
     if (!use_beta && ctl->done) return;
     scale_body(w, v, n, ctl, use_beta, grid_blk());
 }
@@ -470,6 +476,7 @@ template <int NV>
 __global__ void __cluster_dims__(16, 1, 1) __launch_bounds__(kSmallOrthThreads, 1)
 small_orth_kernel(const double *__restrict__ V, const double *__restrict__ w, long n, int m, double *partials, KrylovCtl *ctl,
                   int selective, double *__restrict__ vout) {
+    sim_enter();
     if (ctl->done) return;             // uniform over the cluster: written below, after every CTA has read it
     __shared__ double sh[2][kRedThreads / 32][NVMAX + 1], hs[NVMAX + 1], h2s[NVMAX + 1], nrm;
     cg::cluster_group cl = cg::this_cluster();
@@ -655,6 +662,7 @@ __global__ void cycle_init_kernel(KrylovCtl *ctl) { cycle_init_body(ctl, 0); }
 // so each member's sums are the ones of a launch of its own).  A member whose
 // solve has converged (ctl->active = 0) or whose cycle is done returns at once.
 __device__ __forceinline__ const KMember &member_of(const KMember *M, const int2 *work, VBlk *vb, int count) {
+    sim_enter();
     const int2 wk = work[blockIdx.x];
     vb->id = wk.y;
     vb->count = count;
@@ -662,6 +670,7 @@ __device__ __forceinline__ const KMember &member_of(const KMember *M, const int2
 }
 // a block of the member's reduction grid (as wide as its own launches': nred)
 __device__ __forceinline__ const KMember &member_red(const KMember *M, const int2 *work, VBlk *vb) {
+    sim_enter();
     const int2 wk = work[blockIdx.x];
     const KMember &m = M[wk.x];
     vb->id = wk.y;
@@ -786,17 +795,17 @@ template <int NV>
 struct OrthDispatch {
     static void dots(int nv, cudaStream_t st, const double *V, const double *w, long n, double *part, unsigned int *tk,
                      double *out, const int *done) {
-        if (nv == NV) dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, part, tk, out, done);
+        if (nv == NV) sim_launch(dots_kernel<NV>, sim_red_blocks(n), kRedThreads, st, V, w, n, part, tk, out, done);
         else OrthDispatch<NV - 1>::dots(nv, st, V, w, n, part, tk, out, done);
     }
     static void norm(int nv, cudaStream_t st, const double *V, double *w, long n, int m, double *part, unsigned int *tk,
                      KrylovCtl *ctl, int sel) {
-        if (nv == NV) orth_norm_kernel<NV><<<sim_red_blocks(n), kNormThreads, 0, st>>>(V, w, n, NV - 1, m, part, tk, ctl, sel);
+        if (nv == NV) sim_launch(orth_norm_kernel<NV>, sim_red_blocks(n), kNormThreads, st, V, w, n, NV - 1, m, part, tk, ctl, sel);
         else OrthDispatch<NV - 1>::norm(nv, st, V, w, n, m, part, tk, ctl, sel);
     }
     static void orth(int nv, cudaStream_t st, const double *V, double *w, long n, const double *h, double *part,
                      unsigned int *tk, double *out, const int *done, int sel) {
-        if (nv == NV) orth_dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, h, part, tk, out, done, sel);
+        if (nv == NV) sim_launch(orth_dots_kernel<NV>, sim_red_blocks(n), kRedThreads, st, V, w, n, h, part, tk, out, done, sel);
         else OrthDispatch<NV - 1>::orth(nv, st, V, w, n, h, part, tk, out, done, sel);
     }
     // every pass and the normalisation into V_{nv} (n <= kSmallOrth)
@@ -812,20 +821,20 @@ struct OrthDispatch {
             return true;
         }();
         if (!ok) return cudaErrorNotSupported;
-        small_orth_kernel<NV><<<16, kSmallOrthThreads, 0, st>>>(V, w, n, m, part, ctl, sel, V + (size_t)NV * n);
+        sim_launch(small_orth_kernel<NV>, 16, kSmallOrthThreads, st, V, w, n, m, part, ctl, sel, V + (size_t)NV * n);
         return cudaGetLastError();
     }
     // batched: one launch per pass over every member's virtual blocks
     static void bdots(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred) {
-        if (nv == NV) b_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred);
+        if (nv == NV) sim_launch(b_dots_kernel<NV>, nred, kRedThreads, st, M, wred);
         else OrthDispatch<NV - 1>::bdots(nv, st, M, wred, nred);
     }
     static void borth(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int sel) {
-        if (nv == NV) b_orth_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred, sel);
+        if (nv == NV) sim_launch(b_orth_dots_kernel<NV>, nred, kRedThreads, st, M, wred, sel);
         else OrthDispatch<NV - 1>::borth(nv, st, M, wred, nred, sel);
     }
     static void bnorm(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int m, int sel) {
-        if (nv == NV) b_orth_norm_kernel<NV><<<nred, kNormThreads, 0, st>>>(M, wred, m, sel);
+        if (nv == NV) sim_launch(b_orth_norm_kernel<NV>, nred, kNormThreads, st, M, wred, m, sel);
         else OrthDispatch<NV - 1>::bnorm(nv, st, M, wred, nred, m, sel);
     }
 };
@@ -1033,8 +1042,8 @@ __global__ void diff_norm_kernel(const double *__restrict__ a, const double *__r
 // y = S x: the block-stencil product, then the rate-controlled wells' Schur
 // term -A_pw A_ww^-1 A_wp x (Eq. 16 with the well unknowns eliminated)
 sim_status k_spmv_block(sim_t *s, const double *x, double *y, int bs) {
-    if (s->b == 2) spmv_kernel<2, double><<<sim_blocks(s->N, bs), bs, 0, s->stream>>>(s->gd, s->J, x, y, nullptr);
-    else spmv_kernel<3, double><<<sim_blocks(s->N, bs), bs, 0, s->stream>>>(s->gd, s->J, x, y, nullptr);
+    if (s->b == 2) sim_launch(spmv_kernel<2, double>, sim_blocks(s->N, bs), bs, s->stream, s->gd, s->J, x, y, nullptr);
+    else sim_launch(spmv_kernel<3, double>, sim_blocks(s->N, bs), bs, s->stream, s->gd, s->J, x, y, nullptr);
     SIM_LAUNCHED(s);
     return k_well_op<double>(s, x, y, nullptr);
 }
@@ -1045,11 +1054,11 @@ static sim_status spmv_done(sim_t *s, const void *x, bool xf, double *y, const i
     const int bs = s->tune_spmv;
     const int nb = sim_blocks(s->N, bs);
     if (s->b == 2) {
-        if (xf) spmv_kernel<2, float><<<nb, bs, 0, s->stream>>>(s->gd, s->J, (const float *)x, y, done);
-        else spmv_kernel<2, double><<<nb, bs, 0, s->stream>>>(s->gd, s->J, (const double *)x, y, done);
+        if (xf) sim_launch(spmv_kernel<2, float>, nb, bs, s->stream, s->gd, s->J, (const float *)x, y, done);
+        else sim_launch(spmv_kernel<2, double>, nb, bs, s->stream, s->gd, s->J, (const double *)x, y, done);
     } else {
-        if (xf) spmv_kernel<3, float><<<nb, bs, 0, s->stream>>>(s->gd, s->J, (const float *)x, y, done);
-        else spmv_kernel<3, double><<<nb, bs, 0, s->stream>>>(s->gd, s->J, (const double *)x, y, done);
+        if (xf) sim_launch(spmv_kernel<3, float>, nb, bs, s->stream, s->gd, s->J, (const float *)x, y, done);
+        else sim_launch(spmv_kernel<3, double>, nb, bs, s->stream, s->gd, s->J, (const double *)x, y, done);
     }
     SIM_LAUNCHED(s);
     return xf ? k_well_op<float>(s, (const float *)x, y, done) : k_well_op<double>(s, (const double *)x, y, done);
@@ -1106,7 +1115,7 @@ static sim_status orth_step(sim_t *s, int nv, const int *done) {
     SIM_LAUNCHED(s);
     OrthDispatch<SIM_MAX_M>::norm(nv, s->stream, s->V, s->w, n, s->m, s->red, s->ticket, ctl, s->opt.orth);
     SIM_LAUNCHED(s);
-    scale_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->w, s->V + (size_t)nv * n, n, ctl, 0);
+    sim_launch(scale_kernel, sim_stream_blocks(n), SIM_THREADS, s->stream, s->w, s->V + (size_t)nv * n, n, ctl, 0);
     SIM_LAUNCHED(s);
     return SIM_OK;
 }
@@ -1122,7 +1131,7 @@ static sim_status enqueue_cycle(sim_t *s) {
     const int *done = &ctl->done;
     cycle_init_kernel<<<1, 64, 0, s->stream>>>(ctl);
     SIM_LAUNCHED(s);
-    scale_kernel<<<sim_stream_blocks(n), SIM_THREADS, 0, s->stream>>>(s->r, s->V, n, ctl, 1);
+    sim_launch(scale_kernel, sim_stream_blocks(n), SIM_THREADS, s->stream, s->r, s->V, n, ctl, 1);
     SIM_LAUNCHED(s);
     for (int j = 0; j < m; j++) {
         double *vj = s->V + (size_t)j * n;
@@ -1447,22 +1456,22 @@ static cudaError_t enqueue_batch_cycle(KrylovBatch *kb, cudaStream_t st, int64_t
     const int2 *W = kb->dwork;
     int64_t n = 0;
     b_cycle_init_kernel<<<kb->one_n, 64, 0, st>>>(M, W + kb->one_off); n++;
-    b_scale_kernel<<<kb->red_n, kRedThreads, 0, st>>>(M, W + kb->red_off, 0, 1); n++;
+    sim_launch(b_scale_kernel, kb->red_n, kRedThreads, st, M, W + kb->red_off, 0, 1); n++;
     for (int j = 0; j < kb->m; j++) {
         const int a = cpr_batch_apply(kb->cpr, st, j);
         if (a < 0) return cudaErrorLaunchFailure;
         n += a;
         if (kb->b == 2) {
-            if (kb->zf) b_spmv_kernel<2, float><<<kb->cell_n, SIM_THREADS, 0, st>>>(M, W + kb->cell_off, j, 0);
-            else b_spmv_kernel<2, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(M, W + kb->cell_off, j, 0);
+            if (kb->zf) sim_launch(b_spmv_kernel<2, float>, kb->cell_n, SIM_THREADS, st, M, W + kb->cell_off, j, 0);
+            else sim_launch(b_spmv_kernel<2, double>, kb->cell_n, SIM_THREADS, st, M, W + kb->cell_off, j, 0);
         } else {
-            if (kb->zf) b_spmv_kernel<3, float><<<kb->cell_n, SIM_THREADS, 0, st>>>(M, W + kb->cell_off, j, 0);
-            else b_spmv_kernel<3, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(M, W + kb->cell_off, j, 0);
+            if (kb->zf) sim_launch(b_spmv_kernel<3, float>, kb->cell_n, SIM_THREADS, st, M, W + kb->cell_off, j, 0);
+            else sim_launch(b_spmv_kernel<3, double>, kb->cell_n, SIM_THREADS, st, M, W + kb->cell_off, j, 0);
         }
         OrthDispatch<SIM_MAX_M>::bdots(j + 1, st, M, W + kb->red_off, kb->red_n);
         OrthDispatch<SIM_MAX_M>::borth(j + 1, st, M, W + kb->red_off, kb->red_n, kb->orth);
         OrthDispatch<SIM_MAX_M>::bnorm(j + 1, st, M, W + kb->red_off, kb->red_n, kb->m, kb->orth);
-        b_scale_kernel<<<kb->red_n, kRedThreads, 0, st>>>(M, W + kb->red_off, j + 1, 0);
+        sim_launch(b_scale_kernel, kb->red_n, kRedThreads, st, M, W + kb->red_off, j + 1, 0);
         n += 5;
     }
     *launches = n;
@@ -1566,8 +1575,8 @@ sim_status k_fgmres_batch(KrylovBatch *kb, sim_t *const *ms, int nm, cudaStream_
         b_backsolve_kernel<<<kb->one_n, 32, 0, st>>>(kb->dmem, kb->dwork + kb->one_off);
         if (kb->zf) b_xupdate_kernel<float><<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
         else b_xupdate_kernel<double><<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
-        if (kb->b == 2) b_spmv_kernel<2, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->cell_off, 0, 1);
-        else b_spmv_kernel<3, double><<<kb->cell_n, SIM_THREADS, 0, st>>>(kb->dmem, kb->dwork + kb->cell_off, 0, 1);
+        if (kb->b == 2) sim_launch(b_spmv_kernel<2, double>, kb->cell_n, SIM_THREADS, st, kb->dmem, kb->dwork + kb->cell_off, 0, 1);
+        else sim_launch(b_spmv_kernel<3, double>, kb->cell_n, SIM_THREADS, st, kb->dmem, kb->dwork + kb->cell_off, 0, 1);
         b_resid_kernel<<<kb->red_n, kRedThreads, 0, st>>>(kb->dmem, kb->dwork + kb->red_off);
         b_gather_kernel<<<kb->one_n, 32, 0, st>>>(kb->dmem, kb->dwork + kb->one_off, kb->dout);
         kb->launches += 5;
