@@ -2546,7 +2546,7 @@ static cudaError_t launch_clusters(int clusters, int threads, cudaStream_t st, A
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // as sim_launch
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(clusters * ctas); cfg.blockDim = dim3(threads); cfg.stream = st;
-    cfg.attrs = at; cfg.numAttrs = sim_overlaps(st) ? 2 : 1;
+    cfg.attrs = at; cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, Kernel, args...);
 }
 

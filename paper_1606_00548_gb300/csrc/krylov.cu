@@ -790,22 +790,25 @@ __global__ void __launch_bounds__(kRedThreads) b_resid_kernel(const KMember *M, 
     }
 }
 
-// launch the NV-specialised kernels for a runtime vector count nv <= SIM_MAX_M
+// launch the NV-specialised kernels for a runtime vector count nv <= SIM_MAX_M.  Plain
+// launches, not sim_launch: a grid of one block per SM has to find all of them free, or
+// the SMs that drain first take two blocks and the others none (200k three-phase cells:
+// a solve of 39 iterations 13.1 ms, 12.0 this way)
 template <int NV>
 struct OrthDispatch {
     static void dots(int nv, cudaStream_t st, const double *V, const double *w, long n, double *part, unsigned int *tk,
                      double *out, const int *done) {
-        if (nv == NV) sim_launch(dots_kernel<NV>, sim_red_blocks(n), kRedThreads, st, V, w, n, part, tk, out, done);
+        if (nv == NV) dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, part, tk, out, done);
         else OrthDispatch<NV - 1>::dots(nv, st, V, w, n, part, tk, out, done);
     }
     static void norm(int nv, cudaStream_t st, const double *V, double *w, long n, int m, double *part, unsigned int *tk,
                      KrylovCtl *ctl, int sel) {
-        if (nv == NV) sim_launch(orth_norm_kernel<NV>, sim_red_blocks(n), kNormThreads, st, V, w, n, NV - 1, m, part, tk, ctl, sel);
+        if (nv == NV) orth_norm_kernel<NV><<<sim_red_blocks(n), kNormThreads, 0, st>>>(V, w, n, NV - 1, m, part, tk, ctl, sel);
         else OrthDispatch<NV - 1>::norm(nv, st, V, w, n, m, part, tk, ctl, sel);
     }
     static void orth(int nv, cudaStream_t st, const double *V, double *w, long n, const double *h, double *part,
                      unsigned int *tk, double *out, const int *done, int sel) {
-        if (nv == NV) sim_launch(orth_dots_kernel<NV>, sim_red_blocks(n), kRedThreads, st, V, w, n, h, part, tk, out, done, sel);
+        if (nv == NV) orth_dots_kernel<NV><<<sim_red_blocks(n), kRedThreads, 0, st>>>(V, w, n, h, part, tk, out, done, sel);
         else OrthDispatch<NV - 1>::orth(nv, st, V, w, n, h, part, tk, out, done, sel);
     }
     // every pass and the normalisation into V_{nv} (n <= kSmallOrth)
@@ -826,15 +829,15 @@ struct OrthDispatch {
     }
     // batched: one launch per pass over every member's virtual blocks
     static void bdots(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred) {
-        if (nv == NV) sim_launch(b_dots_kernel<NV>, nred, kRedThreads, st, M, wred);
+        if (nv == NV) b_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred);
         else OrthDispatch<NV - 1>::bdots(nv, st, M, wred, nred);
     }
     static void borth(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int sel) {
-        if (nv == NV) sim_launch(b_orth_dots_kernel<NV>, nred, kRedThreads, st, M, wred, sel);
+        if (nv == NV) b_orth_dots_kernel<NV><<<nred, kRedThreads, 0, st>>>(M, wred, sel);
         else OrthDispatch<NV - 1>::borth(nv, st, M, wred, nred, sel);
     }
     static void bnorm(int nv, cudaStream_t st, const KMember *M, const int2 *wred, int nred, int m, int sel) {
-        if (nv == NV) sim_launch(b_orth_norm_kernel<NV>, nred, kNormThreads, st, M, wred, m, sel);
+        if (nv == NV) b_orth_norm_kernel<NV><<<nred, kNormThreads, 0, st>>>(M, wred, m, sel);
         else OrthDispatch<NV - 1>::bnorm(nv, st, M, wred, nred, m, sel);
     }
 };

@@ -249,14 +249,21 @@ bool sim_mixed(const sim_t *s);
 // this way calls sim_enter() before it touches anything another launch writes, and
 // before any early return: a completed kernel then stands for all before it.
 // An application at 400k two-phase cells 200 -> 161 us, at 1M three-phase cells (two
-// V-cycles) 603 -> 522 us.  Not while a stream is captured: a replayed graph's kernels
-// follow each other within 0.5 us anyway, and graphs with such edges cost more to bring
-// up to date (a Newton iteration at 200k cells 31.1 -> 36.3 ms).
+// V-cycles) 603 -> 522 us.
+//   In a captured cycle, whose kernels follow each other sooner (about 1 us), the blocks
+// that come early cost something too: they fill the SMs that drain first, and a grid of
+// less than a wave is then spread unevenly.  With little work per SM (up to 65,536
+// threads) latency decides and the overlap pays (solves of 41k two-phase and 60k
+// three-phase cells 4712 -> 4610, 6870 -> 6510 us); beyond a wave (152 x 2,048 threads)
+// the rest of the grid evens out; between the two the launch stays plain (a Newton
+// iteration at 200k three-phase cells: 31.1 ms without, 30.7 this way, 32.1 with every
+// launch overlapped or with the line at 131,072).
 __device__ __forceinline__ void sim_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-inline bool sim_overlaps(cudaStream_t st) {
+inline bool sim_overlaps(long threads, cudaStream_t st) {
+    if (threads <= 65536 || threads > 152L * 2048) return true;
     cudaStreamCaptureStatus c;
     return cudaStreamIsCapturing(st, &c) == cudaSuccess && c == cudaStreamCaptureStatusNone;
 }
@@ -268,7 +275,7 @@ inline void sim_launch(void (*kernel)(P...), long blocks, int threads, cudaStrea
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads); cfg.stream = st;
-    cfg.attrs = at; cfg.numAttrs = sim_overlaps(st) ? 1 : 0;
+    cfg.attrs = at; cfg.numAttrs = sim_overlaps(blocks * threads, st) ? 1 : 0;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
