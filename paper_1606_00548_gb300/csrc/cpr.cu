@@ -2757,7 +2757,7 @@ sim_status cpr_apply(sim_t *s, const double *r, void *z, const int *done) {
 //
 // One launch per stage covers every member: the restriction, each V-cycle
 // level's residual / restriction / prolongation / smoothing (a member takes
-// part in the launches of the levels it has), the coarse end (one 8-CTA
+// part in the launches of the levels it has), the coarse end (one 16-CTA
 // cluster per member for its fused coarse levels, or the dense product of its
 // coarsest level) and the three stage-F sweeps.  Block b of a launch takes
 // work[b] = (member, block of the member's rows), reads the member's operands
