@@ -517,6 +517,12 @@ __device__ __forceinline__ long long neg_bits(double a) {
     const long long v = __double_as_longlong(-a);
     return v > 0 && v <= 0x7ff0000000000000LL ? v : 0;
 }
+// the least strong coupling theta mx as such bits; a bound that is no positive number
+// (theta NaN or negative, 0 times infinity) refuses none, as a < bound does in FP64
+__device__ __forceinline__ long long strong_bits(double theta, long long mx) {
+    const double t = theta * __longlong_as_double(mx);
+    return t > 0.0 ? __double_as_longlong(t) : 0;
+}
 
 // the best candidate so far: strength band (binary exponent), then the symmetric
 // hash of the pair, then the smaller index
@@ -587,7 +593,7 @@ __global__ void __launch_bounds__(SIM_THREADS) match_kernel(Mat<double> A, Match
                 mx = max(mx, a[d]);
             }
             if (mx > 0) {
-                const long long lim = __double_as_longlong(theta * __longlong_as_double(mx));
+                const long long lim = strong_bits(theta, mx);
 #pragma unroll
                 for (int d = 1; d < 7; d++)
                     if (a[d] != 0) consider(nbrc(A.g, cc, d), a[d], lim);
@@ -615,7 +621,7 @@ __global__ void __launch_bounds__(SIM_THREADS) match_kernel(Mat<double> A, Match
 #pragma unroll
         for (int o = LANES / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (mx > 0) {
-            const long long lim = __double_as_longlong(theta * __longlong_as_double(mx));
+            const long long lim = strong_bits(theta, mx);
 #pragma unroll
             for (int u = 0; u < U; u++) consider(jj[u], a[u], lim);
             for (int k = sub + LANES * U; k < W; k += LANES) {
