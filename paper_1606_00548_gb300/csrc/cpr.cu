@@ -2118,7 +2118,7 @@ static void *dev_alloc_async(sim_t *s, size_t bytes) {
 static void dev_free_async(sim_t *s, void *p) { if (p) cudaFreeAsync(p, s->stream); }
 
 static void free_level(sim_t *s, AmgLevel &L) {
-    dev_free_async(s, L.work); dev_free_async(s, L.col); dev_free_async(s, L.val);
+    dev_free_async(s, L.work); dev_free_async(s, L.len); dev_free_async(s, L.val);
     dev_free_async(s, L.agg); dev_free_async(s, L.moff); dev_free_async(s, L.mem); dev_free_async(s, L.coarse_inv);
     L = AmgLevel();
 }
@@ -2196,40 +2196,79 @@ static bool enqueue_pass(sim_t *s, const Mat<double> &A, bool second, int *aggC,
     return sim_cuda_ok(s, cudaGetLastError(), "aggregation pass");
 }
 
-// a Galerkin product P^T A P enqueued into fresh ELL arrays of capacity Wcap; its
-// width is read with the next scalars
+// Memory the set-up may write until it returns: the preconditioned directions of the
+// Krylov solver, whose contents no call keeps.  It holds the products while their widths
+// are unknown (48 or 64 slots a row; the longest rows have 19 to 49), so the pool holds
+// the levels at their widths only: 160 B a cell of the pool at 4.2M black-oil cells, 412
+// with the products there too (177 with each width counted by a launch of its own first).
+// What it costs is a copy per large level: 16.8M cells 40.0 -> 40.6 ms, 200k 1556 and
+// 1555 us.
+struct SetupScratch {
+    char *p;
+    size_t size;
+};
+
+// a Galerkin product P^T A P enqueued into ELL arrays of capacity Wcap; its width is
+// read with the next scalars
 struct GalerkinJob {
-    bool on = false;
+    bool on = false, own = false;      // own: arrays of the pool's, else of the scratch
     Mat<double> A;
     const int *agg = nullptr, *moff = nullptr, *mem = nullptr;
     int nc = 0, Wcap = 0, sc = 0;
-    int *col = nullptr;                // Wcap x nc columns, then the nc row lengths
+    SetupScratch scr = {nullptr, 0};   // what it may take of the scratch
+    size_t taken = 0;                  // and took
+    int *len = nullptr;                // row lengths, from ell_head(nc) on the columns
     double *val = nullptr;
-    int *len() const { return col ? col + (size_t)Wcap * nc : nullptr; }
+    int *col() const;
 };
+// ints before the columns in the block of an ELL matrix of n rows
+static size_t ell_head(int n) { return ((size_t)n + 63) & ~(size_t)63; }
+int *GalerkinJob::col() const { return len + ell_head(nc); }
+static size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+static size_t ell_ints(int n, int W) { return up256(sizeof(int) * (ell_head(n) + (size_t)W * n)); }
+static size_t ell_vals(int n, int W) { return up256(sizeof(double) * (size_t)W * n); }
 
+static void galerkin_release(sim_t *s, GalerkinJob &g) {
+    if (g.own) { dev_free_async(s, g.len); dev_free_async(s, g.val); }
+    g.len = nullptr; g.val = nullptr; g.own = false; g.taken = 0;
+}
 static bool galerkin_alloc(sim_t *s, GalerkinJob &g, int W) {
-    dev_free_async(s, g.col); dev_free_async(s, g.val);
+    galerkin_release(s, g);
     g.Wcap = W;
-    g.col = (int *)dev_alloc_async(s, sizeof(int) * (size_t)(W + 1) * g.nc);
-    g.val = (double *)dev_alloc_async(s, sizeof(double) * (size_t)W * g.nc);
-    return g.col && g.val &&
-           sim_cuda_ok(s, cudaMemsetAsync(g.col, 0xff, sizeof(int) * (size_t)W * g.nc, s->stream), "memset") &&
+    const size_t bi = ell_ints(g.nc, W), bv = ell_vals(g.nc, W);
+    if (bi + bv <= g.scr.size) {
+        g.len = (int *)g.scr.p;
+        g.val = (double *)(g.scr.p + bi);
+        g.taken = bi + bv;
+    } else {
+        g.own = true;
+        g.len = (int *)dev_alloc_async(s, bi);
+        g.val = (double *)dev_alloc_async(s, bv);
+        if (!g.len || !g.val) return false;
+    }
+    return sim_cuda_ok(s, cudaMemsetAsync(g.col(), 0xff, sizeof(int) * (size_t)W * g.nc, s->stream), "memset") &&
            sim_cuda_ok(s, cudaMemsetAsync(s->iscal + g.sc, 0, 2 * sizeof(int), s->stream), "memset");
 }
 static bool galerkin_rows(sim_t *s, GalerkinJob &g) {
     galerkin_row_kernel<<<(g.nc + kGalWarps - 1) / kGalWarps, kGalWarps * 32, 0, s->stream>>>(
-        g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col, g.val, g.len(), s->iscal + g.sc, s->iscal + g.sc + 1);
+        g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col(), g.val, g.len, s->iscal + g.sc, s->iscal + g.sc + 1);
     s->launches++;
     return sim_cuda_ok(s, cudaGetLastError(), "Galerkin");
 }
+// scr: the scratch it may take; roomy: the pool may hold its capacity for a while
 static bool enqueue_galerkin(sim_t *s, GalerkinJob &g, const Mat<double> &A, const int *agg, const int *moff, const int *mem,
-                             int nc, int sc) {
+                             int nc, int sc, SetupScratch scr, bool roomy) {
     g = GalerkinJob();
-    g.on = true; g.A = A; g.agg = agg; g.moff = moff; g.mem = mem; g.nc = nc; g.sc = sc;
-    // rows of these hierarchies have 15 to 35 columns; the wider bound costs memory
-    // only, so it is tighter where that is large
-    return galerkin_alloc(s, g, nc <= (1 << 20) ? 64 : 48) && galerkin_rows(s, g);
+    g.on = true; g.A = A; g.agg = agg; g.moff = moff; g.mem = mem; g.nc = nc; g.sc = sc; g.scr = scr;
+    // Rows of these hierarchies have 15 to 49 columns: a product that 40 slots a row do
+    // not hold is rare, and completed by resolve_galerkin.  Where neither the scratch
+    // (few Krylov directions) nor a small level leaves room for that, one slot a row: the
+    // row kernel then counts, and resolve_galerkin builds the product at its width.
+    const int want = nc <= (1 << 20) ? 64 : 48;
+    int W = want;
+    while (W > 40 && ell_ints(nc, W) + ell_vals(nc, W) > scr.size) W--;
+    if (ell_ints(nc, W) + ell_vals(nc, W) > scr.size) W = roomy || nc <= (1 << 17) ? want : 1;
+    return galerkin_alloc(s, g, W) && galerkin_rows(s, g);
 }
 // width of an enqueued product from its scalars; 0: a row wider than SIM_MAX_ELL
 // (the caller stops coarsening), -1: error.  A list the row kernel does not take or
@@ -2248,8 +2287,8 @@ static int resolve_galerkin(sim_t *s, GalerkinJob &g, const int (&v)[kScCount], 
             return -1;
         }
         int u[kScCount];
-        galerkin_kernel<<<sim_blocks(g.nc), SIM_THREADS, 0, s->stream>>>(g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col, g.val,
-                                                                         g.len(), s->iscal + g.sc, s->iscal + g.sc + 1);
+        galerkin_kernel<<<sim_blocks(g.nc), SIM_THREADS, 0, s->stream>>>(g.A, g.agg, g.moff, g.mem, g.nc, g.Wcap, g.col(), g.val,
+                                                                         g.len, s->iscal + g.sc, s->iscal + g.sc + 1);
         s->launches++;
         if (!sim_cuda_ok(s, cudaGetLastError(), "Galerkin") || !read_scalars(s, u)) return -1;
         W = u[g.sc];
@@ -2259,7 +2298,7 @@ static int resolve_galerkin(sim_t *s, GalerkinJob &g, const int (&v)[kScCount], 
 }
 static Mat<double> job_mat(sim_t *s, const GalerkinJob &g) {
     Mat<double> A;
-    A.st = false; A.selfpad = false; A.diff = false; A.g = s->gd; A.n = g.nc; A.width = g.Wcap; A.col = g.col; A.val = g.val; A.len = g.len();
+    A.st = false; A.selfpad = false; A.diff = false; A.g = s->gd; A.n = g.nc; A.width = g.Wcap; A.col = g.col(); A.val = g.val; A.len = g.len;
     A.wp = s->iscal + g.sc;
     return A;
 }
@@ -2268,10 +2307,9 @@ static Mat<double> job_mat(sim_t *s, const GalerkinJob &g) {
 // the ELL levels
 template <typename T>
 static sim_status level_work(sim_t *s, AmgLevel &L, bool ell) {
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t vec = up(sizeof(T) * L.n), colb = ell ? up(sizeof(int) * (size_t)L.width * L.n) : 0;
+    const size_t vec = up256(sizeof(T) * L.n), colb = ell ? up256(sizeof(int) * (size_t)L.width * L.n) : 0;
     const bool copy = ell && sizeof(T) != sizeof(double);     // the FP64 form applies the set-up's values
-    const size_t valb = copy ? up(sizeof(T) * (size_t)L.width * L.n) : 0;
+    const size_t valb = copy ? up256(sizeof(T) * (size_t)L.width * L.n) : 0;
     char *p = (char *)dev_alloc_async(s, 4 * vec + colb + valb);
     if (!p) return s->err;
     L.work = p;
@@ -2349,11 +2387,35 @@ static sim_status finish_levels(sim_t *s) {
     return SIM_OK;
 }
 
-// coarsen from level 0 (whose work vectors the caller has allocated)
-static sim_status amg_setup(sim_t *s) {
+// the product of g at its width W becomes level L's matrix.  Levels of more than
+// kExactRows rows are moved into arrays of that width (one copy each: slots lie row after
+// row); a smaller one keeps its capacity, 7 MB at most beyond its width.
+constexpr int kExactRows = 1 << 14;
+static bool take_product(sim_t *s, GalerkinJob &g, AmgLevel &L, int W) {
+    L.width = W;
+    if (g.own && (W == g.Wcap || g.nc <= kExactRows)) {
+        L.len = g.len; L.val = g.val;
+        g.own = false;
+    } else {
+        L.len = (int *)dev_alloc_async(s, ell_ints(g.nc, W));
+        L.val = (double *)dev_alloc_async(s, ell_vals(g.nc, W));
+        if (!L.len || !L.val ||
+            !sim_cuda_ok(s, cudaMemcpyAsync(L.len, g.len, sizeof(int) * (ell_head(g.nc) + (size_t)W * g.nc),
+                                            cudaMemcpyDeviceToDevice, s->stream), "copy") ||
+            !sim_cuda_ok(s, cudaMemcpyAsync(L.val, g.val, sizeof(double) * (size_t)W * g.nc, cudaMemcpyDeviceToDevice,
+                                            s->stream), "copy"))
+            return false;
+    }
+    L.col = L.len + ell_head(g.nc);
+    galerkin_release(s, g);
+    return true;
+}
+
+// coarsen from level 0 (whose work vectors the caller has allocated); jm: the current
+// level's matrix while its width is unread, j1: the intermediate one it is built from
+static sim_status coarsen(sim_t *s, GalerkinJob &jm, GalerkinJob &j1) {
     const int cmax = s->opt.amg_coarse_max;
-    GalerkinJob jm, j1;                    // the current level's matrix while its width is unread, and its first pass's
-    int *old_col = nullptr; double *old_val = nullptr;   // what jm's product is built from
+    const SetupScratch scr = {(char *)s->Z, (sim_mixed(s) ? sizeof(float) : sizeof(double)) * (size_t)s->m * s->N * s->b};
     int v[kScCount];
     bool rebuilt = false;
     // jm's width arrives with the scalars in v: its level takes it, or the level goes
@@ -2362,20 +2424,18 @@ static sim_status amg_setup(sim_t *s) {
         *gone = rebuilt = false;
         if (!jm.on) return true;
         const int W = resolve_galerkin(s, jm, v, &rebuilt);
-        AmgLevel &L = s->lev.back();
-        L.col = jm.col; L.val = jm.val; L.len = jm.len(); L.width = W;
-        dev_free_async(s, old_col); dev_free_async(s, old_val);      // after a rebuild in stream order
-        old_col = nullptr; old_val = nullptr;
         if (W < 0) return false;
+        galerkin_release(s, j1);                       // after a rebuild in stream order
         if (W == 0) {
-            free_level(s, L);
+            galerkin_release(s, jm);
             s->lev.pop_back();
             AmgLevel &P = s->lev.back();
             dev_free_async(s, P.agg); dev_free_async(s, P.moff); dev_free_async(s, P.mem);
             P.agg = P.moff = P.mem = nullptr;
             *gone = true;
+            return true;
         }
-        return true;
+        return take_product(s, jm, s->lev.back(), W);
     };
     bool gone = false;
     while (true) {
@@ -2389,7 +2449,7 @@ static sim_status amg_setup(sim_t *s) {
         } while (rebuilt && !gone);
         if (gone) break;
         const int n1 = v[kScNc];
-        if (!enqueue_galerkin(s, j1, A, s->aggA, s->moffA, s->memA, n1, kScM1)) return s->err;
+        if (!enqueue_galerkin(s, j1, A, s->aggA, s->moffA, s->memA, n1, kScM1, scr, false)) return s->err;
         AmgLevel &L = s->lev[l];
         L.agg = (int *)dev_alloc_async(s, sizeof(int) * (size_t)n);
         L.moff = (int *)dev_alloc_async(s, sizeof(int) * (size_t)(n1 + 1));
@@ -2411,19 +2471,26 @@ static sim_status amg_setup(sim_t *s) {
         // a row of the intermediate matrix wider than SIM_MAX_ELL, or more than three
         // quarters of the rows left: this level is the coarsest
         if (W1 == 0 || 4L * n2 > 3L * n) {
-            dev_free_async(s, j1.col); dev_free_async(s, j1.val);
+            galerkin_release(s, j1);
             dev_free_async(s, L.agg); dev_free_async(s, L.moff); dev_free_async(s, L.mem);
             L.agg = L.moff = L.mem = nullptr;
             break;
         }
-        if (!enqueue_galerkin(s, jm, A1, s->aggB, s->moffB, s->memB, n2, kScM)) return s->err;
-        old_col = j1.col; old_val = j1.val;
-        AmgLevel C;
-        C.n = n2; C.width = jm.Wcap; C.col = jm.col; C.val = jm.val; C.len = jm.len();
-        s->lev.push_back(C);
+        const bool rest = n2 > kExactRows;             // else the level keeps what it is built in
+        const SetupScratch after = {scr.p + j1.taken, rest ? scr.size - j1.taken : 0};
+        if (!enqueue_galerkin(s, jm, A1, s->aggB, s->moffB, s->memB, n2, kScM, after, !j1.own)) return s->err;
+        s->lev.emplace_back();
+        s->lev.back().n = n2;
     }
     if (jm.on && (!read_scalars(s, v) || !settle(&gone))) return s->err;
-    dev_free_async(s, old_col); dev_free_async(s, old_val);
+    return SIM_OK;
+}
+
+static sim_status amg_setup(sim_t *s) {
+    GalerkinJob jm, j1;
+    const sim_status st = coarsen(s, jm, j1);
+    galerkin_release(s, jm); galerkin_release(s, j1);  // what a failed set-up leaves
+    if (st != SIM_OK) return st;
     if (s->lev.back().n > 1024) return sim_fail(s, SIM_ELIMIT, "AMG coarsest level larger than 1024 rows");
     return sim_mixed(s) ? finish_levels<float>(s) : finish_levels<double>(s);
 }

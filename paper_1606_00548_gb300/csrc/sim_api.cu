@@ -280,7 +280,20 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
     s->mold = (double *)A(sizeof(double) * n);
     s->R = (double *)A(sizeof(double) * n);
     s->J = (double *)A(sizeof(double) * 7 * b * b * N);
-    s->props = (double *)A(sizeof(double) * (b == 2 ? 10 : 21) * N);
+    // the properties live from an assembly's first pass to its second; the integer scratch
+    // of the AMG set-up (68 bytes a cell) shares their memory
+    struct { int **p; size_t n; } scratch[] = {
+        {&s->partner, (size_t)N}, {&s->pick, (size_t)N}, {&s->pick2, (size_t)N}, {&s->absorbed, 6 * (size_t)N},
+        {&s->host, (size_t)N}, {&s->cnt, (size_t)N}, {&s->aggA, (size_t)N}, {&s->aggB, (size_t)N},
+        {&s->moffA, (size_t)N + 1}, {&s->memA, (size_t)N}, {&s->moffB, (size_t)N + 1}, {&s->memB, (size_t)N}};
+    size_t scratch_bytes = 0;
+    for (auto &a : scratch) scratch_bytes += (sizeof(int) * a.n + 255) & ~(size_t)255;
+    s->props = (double *)A(std::max(sizeof(double) * (b == 2 ? 10 : 21) * N, scratch_bytes));
+    size_t at = 0;
+    for (auto &a : scratch) {
+        *a.p = ok ? (int *)((char *)s->props + at) : nullptr;
+        at += (sizeof(int) * a.n + 255) & ~(size_t)255;
+    }
     double *pvt_dev = (double *)A(sizeof(double) * (pvt.size() + 1));
     c.pvt = pvt_dev;
     s->qtot = (double *)A(sizeof(double) * 4);
@@ -316,18 +329,6 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
         s->rhT = A(tsz * n);
         s->x0 = A(tsz * n);
     }
-    s->partner = (int *)A(sizeof(int) * N);
-    s->pick = (int *)A(sizeof(int) * N);
-    s->pick2 = (int *)A(sizeof(int) * N);
-    s->absorbed = (int *)A(sizeof(int) * 6 * N);
-    s->aggA = (int *)A(sizeof(int) * N);
-    s->aggB = (int *)A(sizeof(int) * N);
-    s->host = (int *)A(sizeof(int) * N);
-    s->cnt = (int *)A(sizeof(int) * N);
-    s->moffA = (int *)A(sizeof(int) * (N + 1));
-    s->memA = (int *)A(sizeof(int) * N);
-    s->moffB = (int *)A(sizeof(int) * (N + 1));
-    s->memB = (int *)A(sizeof(int) * N);
     s->scan = (int *)A(sizeof(int) * 3 * (N / 256 + 2));
     s->iscal = (int *)A(sizeof(int) * 16);
     if (!ok) {

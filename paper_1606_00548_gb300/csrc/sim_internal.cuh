@@ -107,8 +107,8 @@ struct BicgCtl {
 
 struct AmgLevel {
     int n = 0, width = 0;        // level 0: width 7, structured
-    int *col = nullptr;          // ELL columns [width][n] (levels >= 1), -1 padding
-    int *len = nullptr;          // entries of each row (behind col in its allocation)
+    int *len = nullptr;          // entries of each row (levels >= 1)
+    int *col = nullptr;          // ELL columns [width][n], -1 padding (behind len in its allocation)
     int *colA = nullptr;         // the same with padding on the row's own column (apply)
     double *val = nullptr;       // ELL values, FP64 (setup precision)
     void *valT = nullptr;        // ELL values in apply precision (float copy for mixed)
@@ -166,7 +166,8 @@ struct sim {
     int8_t *ph = nullptr, *ph_old = nullptr;
     double *mold = nullptr;                  // [b][N]
     double *R = nullptr, *J = nullptr;       // [b][N], [7][b][b][N]
-    double *props = nullptr;                 // [10 (b = 2) or 21][N] densities and mobilities (assemble.cu)
+    double *props = nullptr;                 // [10 (b = 2) or 21][N] densities and mobilities (assemble.cu);
+                                             // between assemblies the AMG set-up's integer scratch
     double *qtot = nullptr;                  // [3] well rates of the last assembly
     double cum_well[3] = {0, 0, 0};
 
@@ -224,7 +225,7 @@ struct sim {
     void *lscT = nullptr;        // [b][b][N] apply precision (aliases lsc in FP64 mode)
     void *rhT = nullptr, *x0 = nullptr;   // [b][N] CPR-FPF: L r - Ahat x0 and the first stage-F result
     std::vector<AmgLevel> lev;
-    // AMG setup scratch
+    // AMG setup scratch (all but scan and iscal lie in props)
     int *partner = nullptr, *pick = nullptr, *pick2 = nullptr, *host = nullptr, *cnt = nullptr, *absorbed = nullptr;
     int *aggA = nullptr, *moffA = nullptr, *memA = nullptr, *aggB = nullptr, *moffB = nullptr, *memB = nullptr;
     int *scan = nullptr, *iscal = nullptr;
