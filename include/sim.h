@@ -149,18 +149,20 @@ typedef struct {
 /* Per-phase figures of a Newton call: device time between CUDA events
    recorded on the handle's stream (microseconds) and the algorithmic bytes of
    the phase, i.e. what its kernels must read and write at least once, from
-   the sizes alone (not measured traffic):
+   the sizes and the matrices' entries (not measured traffic):
      assembly  read x, the step's accumulation, T, porosity; write R, J:
                N (7 b^2 + 3 b + 4) 8
      setup     decoupling reads J, writes Ahat (t bytes per value: 8 FP64,
                4 mixed) and A_p; ILU(0) / block Jacobi reads Ahat, writes the
                inverted diagonal blocks; each coarsening reads its level's
                matrix four times and writes the next level and its map:
-               N (7 b^2 (8 + 2 t) + 7 * 8 + b^2 t) + sum_l (4 w_l n_l 12 + w_{l+1} n_{l+1} 12 + 4 n_l)
+               N (7 b^2 (8 + 2 t) + 7 * 8 + b^2 t) + sum_l (4 e_l 12 + e_{l+1} 12 + 4 n_l)
+               (level l: n_l rows, e_l entries; e_0 = 7 N, a coarse level's
+               rows count the columns they have)
      solve     per FGMRES iteration with basis vectors 0..j: the product
                (7 b^2 + b) 8 N + b N tz (tz: the direction's precision), one
                CPR application (restriction, V-cycle: three passes over each
-               level's matrix, stage F: pressure columns of Ahat, the ILU
+               level's entries, stage F: pressure columns of Ahat, the ILU
                blocks, vectors), the Gram-Schmidt passes (3 (j + 1) + 7) n 8
                (n = b N); per restart the solution update, one product and the
                residual; BiCGSTAB: two products, two applications and 12

@@ -1002,27 +1002,34 @@ __global__ void galerkin_kernel(Mat<double> A, const int *__restrict__ agg, cons
 // What the application reads of the coarse levels, all levels in one launch, a
 // thread per row: 1 / l1 row sums, the columns with padding on the row itself
 // (value 0), and the FP32 copy in the difference form: the diagonal entry replaced
-// by the row sum (computed in FP64), the others rounded as they are.
+// by the row sum (computed in FP64), the others rounded as they are.  It also counts each
+// level's entries (a sum over the warp and one atomic), which the byte models report.
 constexpr int kFinishLevels = 16;
 struct FinishLevel {
     int n, width, row0;          // row0: first row of the level in the launch's row numbering
-    const int *col;
+    const int *col, *len;
     double *val;
     int *colA;
     void *valT, *dinvT;
 };
 struct FinishTable {
     int count, rows;
+    unsigned long long *entries;             // of each level
     FinishLevel lv[kFinishLevels];
 };
 template <typename T>
 __global__ void __launch_bounds__(128) finish_levels_kernel(const __grid_constant__ FinishTable tb) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= tb.rows) return;
     int l = 0;
     while (l + 1 < tb.count && t >= tb.lv[l + 1].row0) l++;
     const FinishLevel &L = tb.lv[l];
     const int i = t - L.row0, n = L.n;
+    const int len = t < tb.rows ? L.len[i] : 0;
+    for (int q = __reduce_min_sync(0xffffffffu, l), q1 = __reduce_max_sync(0xffffffffu, l); q <= q1; q++) {
+        const int c = __reduce_add_sync(0xffffffffu, l == q ? len : 0);
+        if ((threadIdx.x & 31) == 0) atomicAdd(tb.entries + q, (unsigned long long)c);
+    }
+    if (t >= tb.rows) return;
     double s = 0.0, rs = 0.0;
     for (int k0 = 0; k0 < L.width; k0 += 8) {
         int j[8];
@@ -2148,8 +2155,8 @@ static Mat<T> level_matT(sim_t *s, const AmgLevel &L, int l) {
 
 // ---- coarsening -------------------------------------------------------------
 // scalars of the set-up in s->iscal: the aggregate count of the last pass, then
-// {largest row, flags} of the level's matrix and of its intermediate one
-constexpr int kScNc = 0, kScBad = 4, kScM = 8, kScM1 = 10, kScCount = 16;
+// {largest row, flags} of the level's matrix and of its intermediate one; behind them the entry counts (64 bits each) of up to kScLevels levels
+constexpr int kScNc = 0, kScBad = 4, kScM = 8, kScM1 = 10, kScCount = SIM_SETUP_SCALARS, kScLevels = SIM_SETUP_LEVELS;
 
 static bool read_scalars(sim_t *s, int (&v)[kScCount]) {
     if (!sim_cuda_ok(s, cudaMemcpyAsync(s->h_pinned, s->iscal, sizeof(int) * kScCount, cudaMemcpyDeviceToHost, s->stream), "copy") ||
@@ -2325,14 +2332,19 @@ template <typename T>
 static sim_status finish_levels(sim_t *s) {
     // l1 inverse diagonals, apply-precision values, work vectors; coarsest dense inverse
     const int nl = (int)s->lev.size();
+    // the pivot flag and the levels' entry counts come back together
+    int *bad = s->iscal + kScBad;
+    SIM_CK(s, cudaMemsetAsync(bad, 0, sizeof(int) * (kScCount - kScBad + 2 * kScLevels), s->stream));
+    s->lev[0].entries = 7.0 * s->N;
     for (int l0 = 1; l0 < nl; l0 += kFinishLevels) {
         FinishTable tb;
         tb.count = 0; tb.rows = 0;
+        tb.entries = (unsigned long long *)(s->iscal + kScCount) + l0;
         for (int l = l0; l < nl && l < l0 + kFinishLevels; l++) {
             AmgLevel &L = s->lev[l];
             if (level_work<T>(s, L, true) != SIM_OK) return s->err;
             FinishLevel &f = tb.lv[tb.count++];
-            f.n = L.n; f.width = L.width; f.row0 = tb.rows; f.col = L.col; f.val = L.val; f.colA = L.colA; f.valT = L.valT;
+            f.n = L.n; f.width = L.width; f.row0 = tb.rows; f.col = L.col; f.len = L.len; f.val = L.val; f.colA = L.colA; f.valT = L.valT;
             f.dinvT = L.dinvT;
             tb.rows += L.n;
         }
@@ -2346,8 +2358,6 @@ static sim_status finish_levels(sim_t *s) {
     // strongly heterogeneous fields are ill-conditioned, and the product is tiny
     C.coarse_inv = dev_alloc_async(s, sizeof(double) * (size_t)n * n);
     if (!C.coarse_inv) return s->err;
-    int *bad = s->iscal + kScBad;
-    SIM_CK(s, cudaMemsetAsync(bad, 0, sizeof(int), s->stream));
     static bool smem_ok = cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)gj_inverse_bytes(kGjSmem, 8)) == cudaSuccess;
     static int gj_ctas = gj_cluster_ctas();
@@ -2379,10 +2389,12 @@ static sim_status finish_levels(sim_t *s) {
     SIM_CK(s, cudaGetLastError());
     // the pivot test of the elimination (no pivoting: a vanishing pivot would
     // leave inf / NaN in the coarsest inverse)
-    SIM_CK(s, cudaMemcpyAsync(&s->h_pinned[0], bad, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    SIM_CK(s, cudaMemcpyAsync(s->h_pinned, s->iscal, sizeof(int) * (kScCount + 2 * kScLevels), cudaMemcpyDeviceToHost, s->stream));
     SIM_CK(s, cudaStreamSynchronize(s->stream));
     int hb = 0;
-    memcpy(&hb, &s->h_pinned[0], sizeof(int));
+    memcpy(&hb, (const int *)s->h_pinned + kScBad, sizeof(int));
+    const unsigned long long *entries = (const unsigned long long *)((const int *)s->h_pinned + kScCount);
+    for (int l = 1; l < nl; l++) s->lev[l].entries = (double)entries[l];
     if (hb) return sim_fail(s, SIM_ENAN, "coarsest AMG level: a Gauss-Jordan pivot is not above 1e-14 of its row's l1 norm");
     return SIM_OK;
 }

@@ -330,13 +330,13 @@ sim_status sim_create(const sim_grid *g, const sim_rock *r, const sim_fluid *f, 
         s->x0 = A(tsz * n);
     }
     s->scan = (int *)A(sizeof(int) * 3 * (N / 256 + 2));
-    s->iscal = (int *)A(sizeof(int) * 16);
+    s->iscal = (int *)A(sizeof(int) * (SIM_SETUP_SCALARS + 2 * SIM_SETUP_LEVELS));
     if (!ok) {
         std::string m = s->msg;
         sim_destroy(s);
         return sim_fail(nullptr, SIM_ENOMEM, m);
     }
-    if (cudaMallocHost(&s->h_pinned, sizeof(double) * 64) != cudaSuccess ||
+    if (cudaMallocHost(&s->h_pinned, sizeof(double) * 128) != cudaSuccess ||
         cudaMallocHost(&s->ctl_host, sizeof(KrylovCtl)) != cudaSuccess ||
         cudaMallocHost(&s->bctl_host, sizeof(BicgCtl)) != cudaSuccess) {
         sim_destroy(s);
@@ -525,7 +525,7 @@ static sim_status forcing_term(sim_t *s, const Forcing &f, double bnorm, double 
 }
 
 // ---- per-phase figures of a Newton iteration (sim_phase_info) ----------------
-// algorithmic bytes from the sizes alone (the model stated in sim.h)
+// algorithmic bytes from the sizes and the levels' entries (the model stated in sim.h)
 static double apply_bytes_per_value(const sim_t *s) { return sim_mixed(s) ? 4.0 : 8.0; }
 
 static double bytes_assembly(const sim_t *s) {
@@ -540,9 +540,7 @@ static double bytes_setup(const sim_t *s) {
     double v = N * (7 * b * b * (8 + 2 * t) + 7 * 8 + b * b * t);
     const int nl = (int)s->lev.size();
     for (int l = 0; l + 1 < nl; l++) {
-        const double n = s->lev[l].n, w = s->lev[l].width;
-        const double nn = s->lev[l + 1].n, wn = s->lev[l + 1].width;
-        v += 4 * w * n * 12 + wn * nn * 12 + 4 * n;
+        v += 4 * s->lev[l].entries * 12 + s->lev[l + 1].entries * 12 + 4.0 * s->lev[l].n;
     }
     return v;
 }
@@ -556,8 +554,7 @@ static double bytes_apply(const sim_t *s) {
     for (int l = 0; l < nl; l++) {
         const double n = s->lev[l].n;
         if (l + 1 == nl) { v += n * n * 8 + 2 * n * t; break; }   // dense coarsest product
-        const double w = s->lev[l].width;
-        v += 3 * w * n * (l == 0 ? t : 4 + t) + 6 * n * t;      // smoothing, residual, prolongation
+        v += 3 * s->lev[l].entries * (l == 0 ? t : 4 + t) + 6 * n * t;      // smoothing, residual, prolongation
     }
     const double stage_f = N * (8 * b + b * b * t + 7 * b * t + t + b * t)      // r - Ahat x1 (pressure columns)
                          + N * (7 * b * b * t + b * b * t + 3 * b * t + b * t); // red-black ILU(0) sweeps

@@ -25,6 +25,8 @@ struct NvtxRange {
 #define SIM_MAX_ELL 512      // widest coarse AMG row: a wider Galerkin row stops coarsening
 #define SIM_RED_BLOCKS 456   // 3 x 152 SMs: grid of the state's reductions (CNV, masses, finiteness)
 #define SIM_THREADS 256
+#define SIM_SETUP_SCALARS 16 // ints the set-up reads back: counts and flags, then 64-bit entry counts of the levels
+#define SIM_SETUP_LEVELS 80  // a level has at most three quarters of the one above: 68 of them at 2^28 cells
 
 // Reductions of the Krylov solvers over n entries: threads of a block that stream
 // and the blocks of the grid.  One block per SM: the kernels are bound by the FP64
@@ -107,6 +109,7 @@ struct BicgCtl {
 
 struct AmgLevel {
     int n = 0, width = 0;        // level 0: width 7, structured
+    double entries = 0.0;        // sum of the row lengths (level 0: 7 n)
     int *len = nullptr;          // entries of each row (levels >= 1)
     int *col = nullptr;          // ELL columns [width][n], -1 padding (behind len in its allocation)
     int *colA = nullptr;         // the same with padding on the row's own column (apply)
