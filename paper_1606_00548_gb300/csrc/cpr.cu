@@ -1239,8 +1239,13 @@ static size_t gj_inverse_bytes(int n, int nc) {
 
 // CTAs of the Gauss-Jordan cluster: 16 (a non-portable size) when the
 // occupancy query finds room for one such cluster at the largest shared-memory
-// size, else the portable 8; the query launches nothing
+// size, else the portable 8; 0 without that much shared memory; the query launches nothing
 static int gj_cluster_ctas() {
+    if (cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)gj_inverse_bytes(kGjSmem, 8)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
     if (cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         (void)cudaGetLastError();
         return 8;
@@ -2358,10 +2363,9 @@ static sim_status finish_levels(sim_t *s) {
     // strongly heterogeneous fields are ill-conditioned, and the product is tiny
     C.coarse_inv = dev_alloc_async(s, sizeof(double) * (size_t)n * n);
     if (!C.coarse_inv) return s->err;
-    static bool smem_ok = cudaFuncSetAttribute(gj_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)gj_inverse_bytes(kGjSmem, 8)) == cudaSuccess;
-    static int gj_ctas = gj_cluster_ctas();
-    if (smem_ok && n <= kGjSmem) {
+    static PerDevice asked;
+    const int gj_ctas = asked.get(sim_device(), gj_cluster_ctas);
+    if (gj_ctas > 0 && n <= kGjSmem) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2623,7 +2627,8 @@ static int coarse_ctas(void (*kernel)(KArgs...), int threads) {
 }
 template <auto Kernel, typename... Args>
 static cudaError_t launch_clusters(int clusters, int threads, cudaStream_t st, Args... args) {
-    static const int ctas = coarse_ctas(Kernel, threads);      // per kernel: its attributes are its own
+    static PerDevice asked;                                    // per kernel: its attributes are its own
+    const int ctas = asked.get(sim_device(), [&] { return coarse_ctas(Kernel, threads); });
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;

@@ -816,13 +816,14 @@ struct OrthDispatch {
                              int sel) {
         if (nv != NV) return OrthDispatch<NV - 1>::small(nv, st, V, w, n, m, part, ctl, sel);
         // a cluster of 16 is a non-portable size; whether the part takes it is asked once
-        static const bool ok = [] {
+        static PerDevice asked;
+        const int ok = asked.get(sim_device(), [] {
             if (cudaFuncSetAttribute(small_orth_kernel<NV>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
                 (void)cudaGetLastError();
-                return false;
+                return 0;
             }
-            return true;
-        }();
+            return 1;
+        });
         if (!ok) return cudaErrorNotSupported;
         sim_launch(small_orth_kernel<NV>, 16, kSmallOrthThreads, st, V, w, n, m, part, ctl, sel, V + (size_t)NV * n);
         return cudaGetLastError();
@@ -1080,10 +1081,11 @@ sim_status k_norm2(sim_t *s, const double *v, long n, double *out) {
 
 // whether the part schedules the 16-CTA cluster of small_orth_kernel (asked once)
 static bool small_orth_ok() {
-    static const bool ok = [] {
+    static PerDevice asked;
+    return asked.get(sim_device(), [] {
         if (cudaFuncSetAttribute(small_orth_kernel<SIM_MAX_M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
             (void)cudaGetLastError();
-            return false;
+            return 0;
         }
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
@@ -1094,11 +1096,10 @@ static bool small_orth_ok() {
         int c = 0;
         if (cudaOccupancyMaxActiveClusters(&c, small_orth_kernel<SIM_MAX_M>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
-            return false;
+            return 0;
         }
-        return c > 0;
-    }();
-    return ok;
+        return c > 0 ? 1 : 0;
+    }) > 0;
 }
 
 // orthogonalise w against V_0..V_{nv-1}, normalise it into V_nv, column nv - 1 of H

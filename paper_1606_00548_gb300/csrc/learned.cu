@@ -812,13 +812,13 @@ static int tc_bricks(const Dims &d) {
     return ((d.nx + TC_M - 1) / TC_M) * ((d.ny + TC_TY - 1) / TC_TY) * ((d.nz + TC_TZ - 1) / TC_TZ);
 }
 static int tc_grid_sms() {
-    static const int sms = [] {
+    static PerDevice asked;
+    return asked.get(sim_device(), [] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             v = 1;
         return v > 0 ? v : 1;
-    }();
-    return sms;
+    });
 }
 // persistent grid: one CTA per SM (the kernel's shared memory admits no second), at most one per brick
 static int tc_grid(const Dims &d) {
@@ -839,15 +839,15 @@ static int wg_grid(const Dims &d) {
     return nb < two ? nb : two;
 }
 
-// once per process: the convolution needs more than the default 48 KB of shared memory
+// once per device: the convolution needs more than the default 48 KB of shared memory
 static bool tc_attrs() {
-    static const bool ok = [] {
+    static PerDevice asked;
+    return asked.get(sim_device(), [] {
         return cudaFuncSetAttribute(conv_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) == cudaSuccess &&
                cudaFuncSetAttribute(conv_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) == cudaSuccess &&
                cudaFuncSetAttribute(conv_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) == cudaSuccess &&
-               cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM) == cudaSuccess;
-    }();
-    return ok;
+               cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM) == cudaSuccess ? 1 : 0;
+    }) > 0;
 }
 
 // the four layers from act[0] into outf

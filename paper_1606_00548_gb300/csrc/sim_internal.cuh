@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/sim.h"
+#include "per_device.h"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -243,6 +244,8 @@ void *sim_alloc(sim_t *s, size_t bytes);
 void sim_free(sim_t *s, void *p);
 inline int sim_blocks(long n, int t = SIM_THREADS) { long b = (n + t - 1) / t; return (int)(b < 1 ? 1 : b); }
 bool sim_mixed(const sim_t *s);
+// the current device, for PerDevice (outside its range when there is none)
+inline int sim_device() { int d = -1; return cudaGetDevice(&d) == cudaSuccess ? d : -1; }
 
 // ---- launches that overlap the drain of the one before --------------------------
 // A CPR application is a chain of 4 to 45 launches of 2 to 60 us; between two plain
