@@ -2720,10 +2720,6 @@ static sim_status vcycle(sim_t *s, const int *done, T *acc = nullptr) {
                                                                          add ? acc : (T *)L.e2, done, add);
         SIM_LAUNCHED(s);
     }
-    if (acc && lf == 0) {
-        sim_launch(copy_add_kernel<T>, sim_blocks(s->N), SIM_THREADS, s->stream, s->N, (const T *)s->lev[0].e2, acc, 1, done);
-        SIM_LAUNCHED(s);
-    }
     return SIM_OK;
 }
 
