@@ -660,6 +660,7 @@ struct AggPass {
     int *aggC, *moffC, *memC;    // the composite of both passes
     int *csum;                   // [3][chunks] founders, members, fine members per chunk
     int *nc;                     // number of aggregates
+    bool scanned;                // csum holds the sums of the chunks before each (agg_scan_kernel)
 };
 
 // founder i's member count; composite: its fine members too
@@ -717,6 +718,28 @@ __global__ void agg_sizes_kernel(AggPass P, Mat<double> A) {
     }
 }
 
+// csum of very many chunks: each chunk's sum becomes the sum of the chunks before it, by one
+// block (a thread takes a run of chunks)
+__global__ void __launch_bounds__(1024) agg_scan_kernel(AggPass P, Mat<double> A, int chunks) {
+    if (unfinished(A)) return;
+    __shared__ int wsum[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, per = (chunks + 1023) / 1024;
+    const int lo = min(chunks, (int)threadIdx.x * per), hi = min(chunks, lo + per);
+    for (int q = 0; q < 3; q++) {
+        int *c = P.csum + (long)q * chunks, sum = 0;
+#pragma unroll 8
+        for (int k = lo; k < hi; k++) sum += c[k];
+        int x = sum;
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        int b = x - sum;
+        for (int w = 0; w < wid; w++) b += wsum[w];
+        for (int k = lo; k < hi; k++) { const int v = c[k]; c[k] = b; b += v; }
+        __syncthreads();
+    }
+}
+
 // v[0..n) ascending
 __device__ __forceinline__ void sort_ints(int *v, int n) {
     for (int a = 1; a < n; a++) {
@@ -728,7 +751,7 @@ __device__ __forceinline__ void sort_ints(int *v, int n) {
 }
 
 // number the aggregates of this block's chunk (its base: the sum of the chunks
-// before it, added up by every block for itself) and write them
+// before it, added up by every block for itself unless agg_scan_kernel has) and write them
 __global__ void agg_write_kernel(AggPass P, Mat<double> A) {
     if (unfinished(A)) return;
     constexpr int kLocal = 24;
@@ -738,8 +761,12 @@ __global__ void agg_write_kernel(AggPass P, Mat<double> A) {
     agg_counts(P, A, i, t);
     for (int q = 0; q < 3; q++) {
         int b = 0;
-        for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) b += P.csum[q * gridDim.x + k];
-        b = block_sum(b);
+        if (P.scanned) {
+            b = P.csum[q * gridDim.x + blockIdx.x];
+        } else {
+            for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) b += P.csum[q * gridDim.x + k];
+            b = block_sum(b);
+        }
         int x = t[q];                                          // inclusive scan over the block's threads
         for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
         if (lane == 31) wsum[q][wid] = x;
@@ -2198,13 +2225,17 @@ static bool enqueue_pass(sim_t *s, const Mat<double> &A, bool second, int *aggC,
     P.agg = second ? s->aggB : s->aggA; P.moff = second ? s->moffB : s->moffA; P.mem = second ? s->memB : s->memA;
     P.aggC = aggC; P.moffC = moffC; P.memC = memC;
     P.csum = s->scan; P.nc = s->iscal + kScNc;
-    // chunks of 256 nodes spread a small level over the SMs; from 256k nodes chunks
-    // of 1,024 keep the sums every block adds up for its base short
+    // chunks of 256 nodes spread a small level over the SMs; from 256k nodes chunks of 1,024
+    // keep the sums every block adds up for its base short.  Those grow with the square of
+    // the chunks: above 4,096 of them one block scans the sums first (64M nodes: 0.14 ms and
+    // the writing launch 2.13 ms, 8.67 without; 16.8M nodes: 0.05 and 0.63, 1.08 without).
     const int threads = n <= (1 << 18) ? 256 : 1024;
     const int chunks = sim_blocks(n, threads);
+    P.scanned = chunks > 4096;
     agg_sizes_kernel<<<chunks, threads, 0, s->stream>>>(P, A);
+    if (P.scanned) agg_scan_kernel<<<1, 1024, 0, s->stream>>>(P, A, chunks);
     agg_write_kernel<<<chunks, threads, 0, s->stream>>>(P, A);
-    s->launches += 2;
+    s->launches += P.scanned ? 3 : 2;
     return sim_cuda_ok(s, cudaGetLastError(), "aggregation pass");
 }
 
@@ -2213,8 +2244,8 @@ static bool enqueue_pass(sim_t *s, const Mat<double> &A, bool second, int *aggC,
 // are unknown (48 or 64 slots a row; the longest rows have 19 to 49), so the pool holds
 // the levels at their widths only: 160 B a cell of the pool at 4.2M black-oil cells, 412
 // with the products there too (177 with each width counted by a launch of its own first).
-// What it costs is a copy per large level: 16.8M cells 40.0 -> 40.6 ms, 200k 1556 and
-// 1555 us.
+// What it costs is a copy per large level: 0.6 ms of 40 at 16.8M cells, a few us of 1555 at
+// 200k (timed the same).
 struct SetupScratch {
     char *p;
     size_t size;
