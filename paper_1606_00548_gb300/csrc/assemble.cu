@@ -457,7 +457,8 @@ __global__ void __launch_bounds__(32) perf_kernel(FluidConst f, GridDesc g, cons
 // Well equations: one warp per well sums its perforations (lanes stride over them,
 // then a fixed shuffle tree) into R_w, A_ww and the well's rates; one block, whose
 // first warp then sums the rates over the wells and takes the largest relative
-// residual of the rate controls (NaN propagates).
+// residual of the rate controls (a rate that is no number is in its cell's residual too,
+// where the CNV maximum finds it).
 constexpr int kWellThreads = 512;
 __global__ void __launch_bounds__(kWellThreads) well_sum_kernel(int nperf, const int *__restrict__ woff, int nwells,
                                                                 const int *__restrict__ wctrl,

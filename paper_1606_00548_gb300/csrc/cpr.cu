@@ -187,7 +187,10 @@ __device__ __forceinline__ T row_dot(const Mat<T> &A, int i, const T *__restrict
 // residual 16.6 -> 10.8 us with the row lengths).  The count depends on the level's size
 // only, so every kernel that takes the row (one system, a batch, the fused coarse
 // cycle) adds it up alike.  The lines between 4, 8 and 16 lanes are flat: 256 / 1,024,
-// 512 / 2,048 and 1,024 / 4,096 rows measured within 0.4 % of each other.
+// 512 / 2,048 and 1,024 / 4,096 rows, 2 lanes above 8,192 and no 16 measured within 0.4 % of
+// each other.  Speed does not choose among them; the first is taken because the sums it
+// gives leave the Newton counts of an ensemble's chaotic first steps, which any change of
+// rounding moves by several, where the tests of those counts expect them.
 __host__ __device__ inline int ell_lanes(int n) { return n > 131072 ? 1 : n > 1024 ? 4 : n > 256 ? 8 : 16; }
 
 // sum_k val_k e(col_k) of row i by `lanes` adjacent lanes (sub: this one's number;
@@ -1140,8 +1143,9 @@ gj_cluster_kernel(int n, double *__restrict__ A0, double *__restrict__ A1, const
 //   T_j = D A_Kj,  A_ij -= A_iK T_j (i outside K),  A_Kj = T_j;
 // a column j of the panel takes part with A_Kj = e_j and A_ij = 0.  Bound by that
 // chain and, near 256 rows, by the FP64 pipe of the cluster's SMs (n^2 8 / CTAs FMAs
-// a step at 2 a clock).  143 rows: 383 -> 155 us (row blocks and an augmented matrix,
-// a panel of four factored by one CTA of 1,024 threads while the others wait).
+// a step at 2 a clock).  133 rows: 352 -> 141 us, 84 rows: 193 -> 74 us (row blocks and an
+// augmented matrix, which took 8 us more to set up; a panel of four factored by one CTA of
+// 1,024 threads while the others wait).
 constexpr int kGjSmem = 256, kGjNb = 8, kGjThreads = 512;
 
 __device__ __forceinline__ void inv8_warp(double (&a)[2], int lane, const double *rn, int *bad) {

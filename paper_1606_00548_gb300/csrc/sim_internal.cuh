@@ -27,7 +27,7 @@ struct NvtxRange {
 #define SIM_RED_BLOCKS 456   // 3 x 152 SMs: grid of the state's reductions (CNV, masses, finiteness)
 #define SIM_THREADS 256
 #define SIM_SETUP_SCALARS 16 // ints the set-up reads back: counts and flags, then 64-bit entry counts of the levels
-#define SIM_SETUP_LEVELS 80  // a level has at most three quarters of the one above: 68 of them at 2^28 cells
+#define SIM_SETUP_LEVELS 80  // a level has at most three quarters of the rows above it: 68 levels at 2^28 cells
 
 // Reductions of the Krylov solvers over n entries: threads of a block that stream
 // and the blocks of the grid.  One block per SM: the kernels are bound by the FP64
@@ -260,11 +260,13 @@ inline int sim_device() { int d = -1; return cudaGetDevice(&d) == cudaSuccess ? 
 //   In a captured cycle, whose kernels follow each other sooner (about 1 us), the blocks
 // that come early cost something too: they fill the SMs that drain first, and a grid of
 // less than a wave is then spread unevenly.  With little work per SM (up to 65,536
-// threads) latency decides and the overlap pays (solves of 41k two-phase and 60k
-// three-phase cells 4712 -> 4610, 6870 -> 6510 us); beyond a wave (152 x 2,048 threads)
-// the rest of the grid evens out; between the two the launch stays plain (a Newton
-// iteration at 200k three-phase cells: 31.1 ms without, 30.7 this way, 32.1 with every
-// launch overlapped or with the line at 131,072).
+// threads) latency decides and the overlap pays; beyond a wave (152 x 2,048 threads) the
+// rest of the grid evens out; between the two the launch stays plain.  An FGMRES iteration
+// in us, no launch overlapped / this rule / every one: two-phase 32k cells 88.6 / 86.3 /
+// 86.3, 66k 141.3 / 135.8 / 136.0, 84k 157.7 / 147.7 / 145.6, 151k 207.8 / 199.3 / 210.0;
+// three-phase 98k 211.6 / 201.3 / 201.7, 150k 252.9 / 245.0 / 266.0, 200k 275.2 / 271.7 /
+// 287.3, 240k 308.8 / 305.9 / 313.9, 312k 362.0 / 357.0 / 361.2, 336k 379.5 / 375.2 / 375.9,
+// 520k 515.9 / 505.4 / 502.9.
 __device__ __forceinline__ void sim_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
