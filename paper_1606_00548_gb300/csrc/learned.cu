@@ -23,6 +23,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "sim_internal.cuh"
@@ -449,14 +450,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
 // weight gradient: dW[t][ci][co] = sum over cells c of In[c + off(t)][ci] * G[c][co]
 // (mma.sync.m16n8k16 BF16 -> FP32; per tap a 16 x 16 product with the cells
 // as the contraction: too narrow for the 128-row tcgen05 tile).
-// Persistent, two CTAs per SM, bricks of 128 x 1 x WG_TZ cells in runs of up to
-// WG_RUN along y, dealt round-robin, the runs of a ragged last x column after all
-// others.  One thread stages by TMA the brick's input slabs (y-1, y, y+1; lines
-// z0-1 .. z0+WG_TZ; cells x0-8 .. x0+135) and its output-gradient lines, both
-// activation planes each, in the rows of 16 bytes the activations have; a run keeps
-// its slabs in a ring of three and stages one new slab a brick (44 KB of L2 reads
-// instead of 99).  Bound by the legacy tensor path: about 24 clocks per MMA and
-// sub-partition, 27 us for 131 x 67 x 29 cells (28 us with three slabs a brick).
+// Persistent, two CTAs per SM, bricks of 128 x 1 x WG_TZ cells dealt round-robin, those of
+// a ragged last x column after all others.  Per brick one thread stages by TMA the three
+// input slabs (y-1, y, y+1; lines z0-1 .. z0+WG_TZ; cells x0-8 .. x0+135) and the brick's
+// output-gradient lines, both activation planes each, in the rows of 16 bytes the
+// activations have.  Bound by the legacy tensor path: about 24 clocks per MMA and
+// sub-partition.  A layer takes, in us, at 131 x 67 x 29 cells 21, at 128 x 128 x 32 29, at
+// 200 x 180 x 33 64, at 256 x 256 x 64 187.  In runs of up to eight bricks along y that
+// kept two of the three slabs it took 27, 38, 86 and 203: the staging saved is not what
+// bounds it, and runs leave SMs idle at the end.  Without the bias gradient, which then took
+// two launches of its own, and with every 128-cell step of a ragged line: 28, 27, 74, 170.
 // Out-of-grid cells arrive as zeros (bounds fill and x padding), so no cell is masked.  Warp w owns taps w, w+8, w+16, w+24; per
 // 16-cell step it loads the gradient fragment once (ldmatrix.trans: rows are
 // cells) and, per tap, the input fragment of the shifted cells, and issues two
@@ -485,7 +488,7 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t 
 
 __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_constant__ CUtensorMap tin,
                                                                  const __grid_constant__ CUtensorMap tg, Dims d,
-                                                                 int run, int cout, float *__restrict__ part,
+                                                                 int nbricks, int cout, float *__restrict__ part,
                                                                  int *__restrict__ status) {
     extern __shared__ uint8_t wg_raw[];
     __shared__ uint64_t bar;
@@ -494,8 +497,7 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
     uint8_t *sin = wg_raw + ((128u - (smem_addr(wg_raw) & 127u)) & 127u);
     uint8_t *sg = sin + WG_IN;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int gz = (d.nz + WG_TZ - 1) / WG_TZ, gy = (d.ny + run - 1) / run;
-    const int nruns = ((d.nx + TC_M - 1) / TC_M) * gy * gz;
+    const int gz = (d.nz + WG_TZ - 1) / WG_TZ;
     if (tid == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -516,42 +518,35 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
     int it = 0;
     bool in_flight = false;   // thread 0: the current brick's copies were started and not yet waited for
     // tap t of this warp's slot j: where its input fragment of the brick's first cells
-    // lies in a slab (matrices (plane 0, cells 0-7), (1, 0-7), (0, 8-15), (1, 8-15) at
-    // the shifted cells), and the slab (0: y - 1)
+    // lies (matrices (plane 0, cells 0-7), (1, 0-7), (0, 8-15), (1, 8-15) at the shifted cells)
     uint32_t a_off[4];
-    int a_slab[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) {
         const int t = warp + 8 * j, dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-        a_slab[j] = dy + 1;
-        a_off[j] = s_in + (uint32_t)((mat & 1) * WG_IBOX + ((dz + 1) * TC_XS + dx + 8 + (mat >> 1) * 8 + mrow) * 16);
+        a_off[j] = s_in + (uint32_t)(((dy + 1) * 2 + (mat & 1)) * WG_IBOX + ((dz + 1) * TC_XS + dx + 8 + (mat >> 1) * 8 + mrow) * 16);
     }
     const uint32_t g_off = s_g + (uint32_t)((mat >> 1) * WG_GBOX + ((mat & 1) * 8 + mrow) * 16);
-    bool stop = false;
-    for (int c = blockIdx.x; c < nruns && !stop && !*abort; c += gridDim.x) {
-        const int yc = c % gy, bz = (c / gy) % gz, bx = c / (gy * gz);
-        const int x0 = bx * TC_M, z0 = bz * WG_TZ, ya = yc * run, yb = min(d.ny, ya + run);
-        const int xend = min(TC_M, d.nx - x0), zend = min(WG_TZ, d.nz - z0);   // beyond: zero gradients
-        for (int y = ya; y < yb; y++, it++) {
-            if (tid == 0) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                const int s0 = y == ya ? 0 : 2;          // slabs y-1+s0 .. y+1 are new; slab y' lies in slot (y' + 1) mod 3
-                mbar_expect(&bar, (3 - s0) * 2 * WG_IBOX + 2 * WG_GBOX);
-                for (int s = s0; s < 3; s++)
-                    for (int h = 0; h < 2; h++)
-                        tma_load_5d(sin + (((y + s) % 3) * 2 + h) * WG_IBOX, &tin, 0, x0 / 8 - 1, y - 1 + s, z0 - 1, h, &bar);
-                for (int h = 0; h < 2; h++) tma_load_5d(sg + h * WG_GBOX, &tg, 0, x0 / 8, y, z0, h, &bar);
-                in_flight = true;
-            }
-            const bool ok = mbar_wait(&bar, it & 1, abort, status, 16);
-            if (tid == 0 && ok) in_flight = false;
-            stop = __syncthreads_or(!ok) != 0;
-            if (stop) break;   // every thread leaves together: no barrier below waits on one that left
-            uint32_t abase[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) abase[j] = a_off[j] + (uint32_t)((y + a_slab[j]) % 3) * (2 * WG_IBOX);
-            for (int zo = 0; zo < zend; zo++) {
-                for (int xk = 0; xk < xend; xk += 16) {
+    for (int br = blockIdx.x; br < nbricks && !*abort; br += gridDim.x, it++) {
+        const int y = br % d.ny, r = br / d.ny, bz = r % gz, bx = r / gz;
+        const int x0 = bx * TC_M, z0 = bz * WG_TZ;
+        if (tid == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_expect(&bar, WG_IN + 2 * WG_GBOX);
+            for (int s = 0; s < 3; s++)
+                for (int h = 0; h < 2; h++)
+                    tma_load_5d(sin + (s * 2 + h) * WG_IBOX, &tin, 0, x0 / 8 - 1, y - 1 + s, z0 - 1, h, &bar);
+            for (int h = 0; h < 2; h++) tma_load_5d(sg + h * WG_GBOX, &tg, 0, x0 / 8, y, z0, h, &bar);
+            in_flight = true;
+        }
+        const bool ok = mbar_wait(&bar, it & 1, abort, status, 16);
+        if (tid == 0 && ok) in_flight = false;
+        if (__syncthreads_or(!ok)) break;   // every thread leaves together: no barrier below waits on one that left
+        // lines zend and 16-cell steps up to xend; beyond them the gradients are zero.  A whole
+        // brick has constant bounds (FULL) and a layer of more than eight outputs both MMAs (WIDE)
+        auto products = [&](auto FULL, auto WIDE, int xend, int zend) {
+            constexpr bool full = decltype(FULL)::value, wide = decltype(WIDE)::value;
+            for (int zo = 0; zo < (full ? WG_TZ : zend); zo++) {
+                for (int xk = 0; xk < (full ? TC_M : xend); xk += 16) {
                     // gradient fragment (B, 16 cells x 16 outputs): matrices (plane 0, cells 0-7), (0, 8-15), (1, 0-7), (1, 8-15)
                     uint32_t b[4];
                     ldsm_x4_t(g_off + (uint32_t)((zo * TC_M + xk) * 16), b[0], b[1], b[2], b[3]);
@@ -561,16 +556,20 @@ __global__ void __launch_bounds__(WG_THREADS, 2) wgrad_tc_kernel(const __grid_co
                         if (t >= WG_TAPS) continue;
                         uint32_t a[4];
                         if (t < 27)
-                            ldsm_x4_t(abase[j] + (uint32_t)((zo * TC_XS + xk) * 16), a[0], a[1], a[2], a[3]);
+                            ldsm_x4_t(a_off[j] + (uint32_t)((zo * TC_XS + xk) * 16), a[0], a[1], a[2], a[3]);
                         else
                             a[0] = a[1] = a[2] = a[3] = 0x3f803f80u;   // BF16 ones
                         mma_bf16(acc[j][0], a[0], a[1], a[2], a[3], b[0], b[1]);
-                        if (cout > 8) mma_bf16(acc[j][1], a[0], a[1], a[2], a[3], b[2], b[3]);
+                        if (wide) mma_bf16(acc[j][1], a[0], a[1], a[2], a[3], b[2], b[3]);
                     }
                 }
             }
-            __syncthreads();   // every warp is done with the buffers before the next brick's copies
-        }
+        };
+        const int xend = min(TC_M, d.nx - x0), zend = min(WG_TZ, d.nz - z0);
+        if (cout <= 8) products(std::false_type(), std::false_type(), xend, zend);
+        else if (xend == TC_M && zend == WG_TZ) products(std::true_type(), std::true_type(), xend, zend);
+        else products(std::false_type(), std::true_type(), xend, zend);
+        __syncthreads();   // every warp is done with the buffers before the next brick's copies
     }
     if (tid == 0 && in_flight && !mbar_drain(&bar, it & 1)) atomicOr(status, 16);
     // partial of this CTA: [28][16 ci][16 co]
@@ -826,16 +825,10 @@ static int tc_grid(const Dims &d) {
     return nb < sms ? nb : sms;
 }
 
-// weight gradient: the longest run of bricks along y that still gives every CTA one,
-// and the persistent grid, two CTAs per SM, at most one per run
-constexpr int WG_RUN = 8;
-static int wg_columns(const Dims &d) { return ((d.nx + TC_M - 1) / TC_M) * ((d.nz + WG_TZ - 1) / WG_TZ); }
-static int wg_run(const Dims &d) {
-    const int r = (int)((long)wg_columns(d) * d.ny / (2 * tc_grid_sms()));
-    return r < 1 ? 1 : r < WG_RUN ? r : WG_RUN;
-}
+static int wg_bricks(const Dims &d) { return ((d.nx + TC_M - 1) / TC_M) * d.ny * ((d.nz + WG_TZ - 1) / WG_TZ); }
+// persistent weight-gradient grid: two CTAs per SM, at most one per brick
 static int wg_grid(const Dims &d) {
-    const int run = wg_run(d), nb = wg_columns(d) * ((d.ny + run - 1) / run), two = 2 * tc_grid_sms();
+    const int nb = wg_bricks(d), two = 2 * tc_grid_sms();
     return nb < two ? nb : two;
 }
 
@@ -885,7 +878,7 @@ static sim_status net_backward(sim_net_t *n, const float *target) {
     uint32_t *gcur = n->g0, *gnext = n->g1;
     for (int l = NLAYER - 1; l >= 0; l--) {
         const int gi = gcur == n->g0 ? 0 : 1;
-        wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[gi], n->d, wg_run(n->d),
+        wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[gi], n->d, wg_bricks(n->d),
                                                                        COUT[l], n->wpart, n->dstat);
         NET_LAUNCHED(n);
         wgrad_fold_kernel<<<sim_blocks(27 * CIN[l] * COUT[l] + COUT[l], 32), 256, 0, n->stream>>>(
@@ -1090,7 +1083,7 @@ sim_status sim_net_time_conv(sim_net_t *n, int32_t which, int32_t reps, double *
                 nullptr, n->dstat, -1);
         } else if (which == 1) {
             wgrad_tc_kernel<<<n->wg_ctas, WG_THREADS, WG_SMEM, n->stream>>>(n->map_win[l], n->map_wg[0], n->d,
-                                                                           wg_run(n->d), COUT[l], n->wpart, n->dstat);
+                                                                           wg_bricks(n->d), COUT[l], n->wpart, n->dstat);
             n->launches++;
             wgrad_fold_kernel<<<sim_blocks(27 * CIN[l] * COUT[l] + COUT[l], 32), 256, 0, n->stream>>>(
                 n->wg_ctas, CIN[l], COUT[l], n->wpart, n->grad + n->off_w[l]);
