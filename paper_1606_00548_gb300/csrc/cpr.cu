@@ -1143,9 +1143,9 @@ gj_cluster_kernel(int n, double *__restrict__ A0, double *__restrict__ A1, const
 //   T_j = D A_Kj,  A_ij -= A_iK T_j (i outside K),  A_Kj = T_j;
 // a column j of the panel takes part with A_Kj = e_j and A_ij = 0.  Bound by that
 // chain and, near 256 rows, by the FP64 pipe of the cluster's SMs (n^2 8 / CTAs FMAs
-// a step at 2 a clock).  133 rows: 352 -> 141 us, 84 rows: 193 -> 74 us (row blocks and an
-// augmented matrix, which took 8 us more to set up; a panel of four factored by one CTA of
-// 1,024 threads while the others wait).
+// a step at 2 a clock).  236 rows: 796 -> 392 us, 133: 352 -> 141, 84: 193 -> 74 (row blocks
+// and an augmented matrix, which took 8 us more to set up; a panel of four factored by one
+// CTA of 1,024 threads while the others wait).
 constexpr int kGjSmem = 256, kGjNb = 8, kGjThreads = 512;
 
 __device__ __forceinline__ void inv8_warp(double (&a)[2], int lane, const double *rn, int *bad) {
