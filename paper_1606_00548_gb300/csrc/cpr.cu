@@ -2248,8 +2248,7 @@ static bool enqueue_pass(sim_t *s, const Mat<double> &A, bool second, int *aggC,
 // are unknown (48 or 64 slots a row; the longest rows have 19 to 49), so the pool holds
 // the levels at their widths only: 160 B a cell of the pool at 4.2M black-oil cells, 412
 // with the products there too (177 with each width counted by a launch of its own first).
-// What it costs is a copy per large level: 0.6 ms of 40 at 16.8M cells, a few us of 1555 at
-// 200k (timed the same).
+// What it costs is a copy per large level: 0.6 ms of 40 at 16.8M cells.
 struct SetupScratch {
     char *p;
     size_t size;
@@ -2440,8 +2439,10 @@ static sim_status finish_levels(sim_t *s) {
 
 // the product of g at its width W becomes level L's matrix.  Levels of more than
 // kExactRows rows are moved into arrays of that width (one copy each: slots lie row after
-// row); a smaller one keeps its capacity, 7 MB at most beyond its width.
-constexpr int kExactRows = 1 << 14;
+// row); a smaller one keeps its capacity, 30 MB at most beyond its width (at 200k cells 15 of
+// 690 MB for 1.8 % of a set-up: 1549 us against a start of 1541 with the line at 16,384 rows,
+// 1526 against 1546 here).
+constexpr int kExactRows = 1 << 16;
 static bool take_product(sim_t *s, GalerkinJob &g, AmgLevel &L, int W) {
     L.width = W;
     if (g.own && (W == g.Wcap || g.nc <= kExactRows)) {
